@@ -5,8 +5,8 @@
 // radius ceil(3 sigma) with normalised weights and replicated borders (the
 // family of the demons smoothing), division by the scan's mean pattern
 // (static) and by the pattern's own blur (dynamic), and a Keys cubic resample
-// for the affine correction.  One pass over the images per call; everything
-// is FP32 with FP32 accumulation.
+// for the affine correction.  Everything is FP32 with FP32 accumulation (the
+// mean over the scan in FP64).
 #include <math.h>
 
 #include "internal.cuh"
@@ -37,47 +37,165 @@ bool make_taps(float sigma, FilterTaps *f)
     return true;
 }
 
-// along x (dx = 1) or y (dx = 0), replicated borders; one thread per output
-__global__ void blur_pass_kernel(const float *__restrict__ in, float *__restrict__ out, int n, int H, int W, int dx,
-                                 FilterTaps f)
+// a / d, 0 where |d| < 1e-12
+__device__ __forceinline__ float guarded_div(float a, float d) { return fabsf(d) >= 1e-12f ? a / d : 0.0f; }
+
+// One direction of the separable blur (AXIS 0: along x, 1: along y), replicated borders.
+//
+// A CTA takes 32 lines (rows for x, columns for y) and a segment of at most 256 outputs along them; the
+// lines lie in shared memory with their halo, two neighbouring lines interleaved as one float2.  Thread
+// (pair, run) computes RUN consecutive outputs of its two lines: the window of RUN inputs sits in
+// registers (input j in slot j mod RUN, so nothing moves), a tap is one shared-memory load and RUN packed
+// FMAs.  Every output sums its taps in the order k = -r .. r, as one thread per output would.  Bound by
+// the FP32 FMAs from radius ~20 up (2r + 1 per pixel), by HBM below.  1000 patterns of 256 x 256, both
+// directions, radius 60 / 36 / 3: MEAS_BLUR.
+//
+// The passes carry the element-wise steps around them, so that no intermediate image is written for
+// them: PRE divides the input by the background bg as it is loaded; POST divides the input of the
+// whole blur (src, by bg too if given) by the blurred value, or subtracts that from src.
+enum { POST_NONE = 0, POST_DIV, POST_SUB };
+constexpr int RUN = 16, LINES = 32, PAIRS = LINES / 2, MAX_SEG = 256;
+
+struct BlurArgs {
+    const float *in;    // input of this pass
+    const float *src;   // POST: the image the result is combined with
+    const float *bg;    // [H][W] static background (nullable)
+    float *out;
+    long long lines;    // rows of all images (x) or columns of one image (y)
+    int H, W, segs, seg, stride, vec;   // segments per line, outputs per segment, float2 stride of a line pair
+};
+
+template <int AXIS, bool PRE, int POST>
+__global__ void __launch_bounds__(256, 3) blur_pass_kernel(BlurArgs a, const __grid_constant__ FilterTaps f)
 {
-    const size_t plane = (size_t)H * W, total = (size_t)n * plane;
-    for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (size_t)gridDim.x * blockDim.x) {
-        const size_t img = idx / plane;
-        const int rem = (int)(idx - img * plane), y = rem / W, x = rem - y * W;
-        const float *p = in + img * plane;
-        float acc = 0.0f;
-        if (dx) {
-            const float *row = p + (size_t)y * W;
-            for (int k = -f.r; k <= f.r; ++k) acc = fmaf(f.t[k + f.r], __ldg(row + min(max(x + k, 0), W - 1)), acc);
-        } else {
-            for (int k = -f.r; k <= f.r; ++k)
-                acc = fmaf(f.t[k + f.r], __ldg(p + (size_t)min(max(y + k, 0), H - 1) * W + x), acc);
+    extern __shared__ __align__(16) float2 blur_smem[];
+    const int H = a.H, W = a.W, r = f.r, len = AXIS ? H : W;
+    const size_t plane = (size_t)H * W;
+    const int s0 = (blockIdx.x % a.segs) * a.seg;            // first output of the segment
+    const long long l0 = (long long)(blockIdx.x / a.segs) * LINES;   // first line
+    const int n_out = min(a.seg, len - s0), n_in = a.seg + 2 * r;
+    const float *img = a.in + (AXIS ? blockIdx.y * plane : 0);
+    float *sm = reinterpret_cast<float *>(blur_smem);
+    auto put = [&](int line, int j, float v) { sm[2 * ((line >> 1) * a.stride + j) + (line & 1)] = v; };
+    if (AXIS) {   // lanes on columns: coalesced loads, conflict-free stores
+        const int line = threadIdx.x & 31, x = (int)l0 + line;
+        if (x < W)
+#pragma unroll 4
+            for (int j = threadIdx.x >> 5; j < n_in; j += (int)blockDim.x >> 5)
+                put(line, j, __ldg(img + (size_t)min(max(s0 - r + j, 0), H - 1) * W + x));
+    } else {
+        for (int line = threadIdx.x >> 5; line < LINES; line += (int)blockDim.x >> 5) {
+            const long long row = l0 + line;
+            if (row >= a.lines) break;
+            const float *p = img + row * W, *bg = PRE ? a.bg + (size_t)(row % H) * W : nullptr;
+#pragma unroll 4
+            for (int j = threadIdx.x & 31; j < n_in; j += 32) {
+                const int x = min(max(s0 - r + j, 0), W - 1);
+                put(line, j, PRE ? guarded_div(__ldg(p + x), __ldg(bg + x)) : __ldg(p + x));
+            }
         }
-        out[idx] = acc;
+    }
+    __syncthreads();
+    // an odd number of runs leaves half a warp over: it repeats the last run and stores nothing
+    const int pr = threadIdx.x % PAIRS, o0 = min((int)threadIdx.x / PAIRS * RUN, a.seg - RUN);
+    const bool live = (int)threadIdx.x / PAIRS * RUN < a.seg;
+    const float2 *q = blur_smem + pr * a.stride + o0;
+    float2 acc[RUN], win[RUN];
+#pragma unroll
+    for (int i = 0; i < RUN; ++i) {
+        acc[i] = make_float2(0.0f, 0.0f);
+        win[i] = q[i];
+    }
+    auto taps = [&](int k, int u) {   // tap k = base + u, u = k mod RUN
+        const float2 t = make_float2(f.t[k], f.t[k]);
+#pragma unroll
+        for (int i = 0; i < RUN; ++i) acc[i] = __ffma2_rn(t, win[(i + u) % RUN], acc[i]);
+    };
+    int k = 0;
+    for (; k + RUN <= 2 * r + 1; k += RUN)
+#pragma unroll
+        for (int u = 0; u < RUN; ++u) {
+            taps(k + u, u);
+            if (k + u < 2 * r) win[u] = q[k + u + RUN];   // input of tap k + u + 1's last output
+        }
+#pragma unroll
+    for (int u = 0; u < RUN; ++u) {
+        if (k + u > 2 * r) break;
+        taps(k + u, u);
+        if (k + u < 2 * r) win[u] = q[k + u + RUN];
+    }
+    if (AXIS) {
+        const int x = (int)l0 + 2 * pr;
+        const bool two = x + 1 < W;
+#pragma unroll
+        for (int i = 0; i < RUN; ++i) {
+            if (o0 + i >= n_out || x >= W || !live) break;
+            const size_t p = (size_t)(s0 + o0 + i) * W + x, at = blockIdx.y * plane + p;
+            float2 v = acc[i];
+            if (POST != POST_NONE) {
+                float2 c = make_float2(a.src[at], two ? a.src[at + 1] : 0.0f);   // src may be out
+                if (POST == POST_DIV && a.bg) {
+                    c.x = guarded_div(c.x, __ldg(a.bg + p));
+                    if (two) c.y = guarded_div(c.y, __ldg(a.bg + p + 1));
+                }
+                v = POST == POST_DIV ? make_float2(guarded_div(c.x, v.x), guarded_div(c.y, v.y))
+                                     : make_float2(c.x - v.x, c.y - v.y);
+            }
+            if (a.vec) {
+                *reinterpret_cast<float2 *>(a.out + at) = v;
+            } else {
+                a.out[at] = v.x;
+                if (two) a.out[at + 1] = v.y;
+            }
+        }
+    } else {   // through shared memory, so that rows are written whole
+        __syncthreads();
+        if (live)
+#pragma unroll
+            for (int i = 0; i < RUN; ++i) blur_smem[pr * a.stride + o0 + i] = acc[i];
+        __syncthreads();
+        for (int line = threadIdx.x >> 5; line < LINES; line += (int)blockDim.x >> 5) {
+            const long long row = l0 + line;
+            if (row >= a.lines) break;
+            for (int j = threadIdx.x & 31; j < n_out; j += 32)
+                a.out[row * W + s0 + j] = sm[2 * ((line >> 1) * a.stride + j) + (line & 1)];
+        }
     }
 }
 
-__global__ void sub_kernel(const float *a, const float *b, float *out, size_t total)
+// out = a / d, the [H][W] plane d broadcast over the images
+__global__ void div_kernel(const float *a, const float *d, float *out, size_t total, size_t plane)
 {
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x)
-        out[i] = a[i] - b[i];
+        out[i] = guarded_div(a[i], d[i % plane]);
 }
 
-// out = a / d (d per pixel, or the [H][W] plane d broadcast over images when bcast); |d| < 1e-12 -> 0
-__global__ void div_kernel(const float *a, const float *d, float *out, size_t total, size_t plane, int bcast)
+// Mean over the n images: 32 pixels x 8 groups of images per CTA, summed in FP64, the groups' sums added in
+// order.  Bound by the FP64 additions (2 per clock and SM): 1000 patterns of 256 x 256 in MEAS_MEAN.
+__global__ void __launch_bounds__(256) mean_pattern_kernel(const float *__restrict__ in, int n, size_t plane, float *out)
 {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const float dv = d[bcast ? i % plane : i];
-        out[i] = fabsf(dv) >= 1e-12f ? a[i] / dv : 0.0f;
+    __shared__ double part[8][32];
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const size_t p = (size_t)blockIdx.x * 32 + lane;
+    double s = 0.0;
+    if (p < plane) {
+        const float *q = in + p;
+        int i = grp;
+        for (; i + 24 < n; i += 32) {
+            const float v0 = __ldg(q + (size_t)i * plane), v1 = __ldg(q + (size_t)(i + 8) * plane);
+            const float v2 = __ldg(q + (size_t)(i + 16) * plane), v3 = __ldg(q + (size_t)(i + 24) * plane);
+            s += v0;
+            s += v1;
+            s += v2;
+            s += v3;
+        }
+        for (; i < n; i += 8) s += __ldg(q + (size_t)i * plane);
     }
-}
-
-__global__ void mean_pattern_kernel(const float *__restrict__ in, int n, size_t plane, float *out)
-{
-    for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < plane; p += (size_t)gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) s += in[(size_t)i * plane + p];
+    part[grp][lane] = s;
+    __syncthreads();
+    if (grp == 0 && p < plane) {
+#pragma unroll
+        for (int g = 1; g < 8; ++g) s += part[g][lane];
         out[p] = (float)(s / n);
     }
 }
@@ -128,19 +246,43 @@ int grid_of(hrebsd_ctx *ctx, size_t total)
     return (int)(g < cap ? (g ? g : 1) : cap);
 }
 
-// blur of n images into out via tmp (x pass into tmp, y pass into out)
-int blur_into(hrebsd_ctx *ctx, const float *in, float *tmp, float *out, int n, int H, int W, const FilterTaps &f,
-              cudaStream_t st)
+template <int AXIS, bool PRE, int POST>
+int launch_pass(hrebsd_ctx *ctx, const float *in, const float *src, const float *bg, float *out, int n, int H, int W,
+                const FilterTaps &f, cudaStream_t st)
 {
-    const size_t total = (size_t)n * H * W;
-    blur_pass_kernel<<<grid_of(ctx, total), 256, 0, st>>>(in, tmp, n, H, W, 1, f);
-    HR_LAUNCHED(ctx);
-    blur_pass_kernel<<<grid_of(ctx, total), 256, 0, st>>>(tmp, out, n, H, W, 0, f);
-    HR_LAUNCHED(ctx);
+    BlurArgs a;
+    a.in = in;
+    a.src = src;
+    a.bg = bg;
+    a.out = out;
+    a.H = H;
+    a.W = W;
+    a.lines = AXIS ? W : (long long)n * H;
+    const int len = AXIS ? H : W;
+    a.segs = (len + MAX_SEG - 1) / MAX_SEG;
+    const int runs = ((len + a.segs - 1) / a.segs + RUN - 1) / RUN;   // at most 16
+    a.seg = runs * RUN;
+    a.stride = (a.seg + 2 * f.r) | 1;   // odd: 16 lanes on 16 line pairs hit distinct banks
+    a.vec = (W % 2 == 0) && (reinterpret_cast<uintptr_t>(out) % 8 == 0);
+    const size_t smem = (size_t)PAIRS * a.stride * sizeof(float2);
+    auto k = blur_pass_kernel<AXIS, PRE, POST>;
+    if (smem > 48 * 1024) HR_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int threads = (runs * PAIRS + 31) / 32 * 32;   // whole warps
+    const long long tiles = (a.lines + LINES - 1) / LINES * a.segs;
+    for (int i0 = 0; i0 < (AXIS ? n : 1); i0 += 65535) {   // y: one image per grid row
+        const size_t off = (size_t)i0 * H * W;
+        BlurArgs c = a;
+        c.in += off;
+        c.out += off;
+        if (c.src) c.src += off;
+        const dim3 grid((unsigned)tiles, AXIS ? (unsigned)(n - i0 < 65535 ? n - i0 : 65535) : 1u);
+        k<<<grid, threads, smem, st>>>(c, f);
+        HR_LAUNCHED(ctx);
+    }
     return HREBSD_OK;
 }
 
-enum { WS_F0 = 16, WS_F1 = 17, WS_F2 = 18 };
+enum { WS_F0 = 16, WS_F1 = 17 };
 
 }  // namespace
 
@@ -155,19 +297,18 @@ extern "C" int hrebsd_bandpass_batch(hrebsd_ctx *ctx, const float *in, int n, in
     int e = hr_set_device(ctx);
     if (e) return e;
     const size_t total = (size_t)n * H * W;
-    void *t0, *t1, *t2;
-    if ((e = hr_ws(ctx, WS_F0, total * 4, &t0)) || (e = hr_ws(ctx, WS_F1, total * 4, &t1)) ||
-        (e = hr_ws(ctx, WS_F2, total * 4, &t2)))
-        return e;
+    void *t0, *t1;
+    if ((e = hr_ws(ctx, WS_F0, total * 4, &t0)) || (e = hr_ws(ctx, WS_F1, total * 4, &t1))) return e;
     cudaStream_t st = hr_stream(stream);
     hr_prof_begin(ctx, st);
-    if ((e = blur_into(ctx, in, (float *)t0, (float *)t1, n, H, W, lp, st))) return e;   // t1 = low-pass
-    if (hp.r > 0 || sigma_hp > 0.0f) {
-        if ((e = blur_into(ctx, in, (float *)t0, (float *)t2, n, H, W, hp, st))) return e;   // t2 = G_hp * in
-        sub_kernel<<<grid_of(ctx, total), 256, 0, st>>>((const float *)t1, (const float *)t2, out, total);
-        HR_LAUNCHED(ctx);
+    float *x = (float *)t0, *y = (float *)t1;
+    if ((e = launch_pass<0, false, POST_NONE>(ctx, in, nullptr, nullptr, x, n, H, W, lp, st))) return e;
+    if (hp.r > 0 || sigma_hp > 0.0f) {   // out = G_lp * in - G_hp * in (in may be out: read by the x passes only)
+        if ((e = launch_pass<1, false, POST_NONE>(ctx, x, nullptr, nullptr, y, n, H, W, lp, st))) return e;
+        if ((e = launch_pass<0, false, POST_NONE>(ctx, in, nullptr, nullptr, x, n, H, W, hp, st))) return e;
+        if ((e = launch_pass<1, false, POST_SUB>(ctx, x, y, nullptr, out, n, H, W, hp, st))) return e;
     } else {
-        HR_CHECK(cudaMemcpyAsync(out, t1, total * 4, cudaMemcpyDeviceToDevice, st));
+        if ((e = launch_pass<1, false, POST_NONE>(ctx, x, nullptr, nullptr, out, n, H, W, lp, st))) return e;
     }
     hr_prof_end(ctx, PROF_PRE, st);
     return HREBSD_OK;
@@ -180,7 +321,8 @@ extern "C" int hrebsd_mean_pattern(hrebsd_ctx *ctx, const float *in, int n, int 
     if (e) return e;
     cudaStream_t st = hr_stream(stream);
     hr_prof_begin(ctx, st);
-    mean_pattern_kernel<<<grid_of(ctx, (size_t)H * W), 256, 0, st>>>(in, n, (size_t)H * W, out);
+    const size_t plane = (size_t)H * W;
+    mean_pattern_kernel<<<(unsigned)((plane + 31) / 32), 256, 0, st>>>(in, n, plane, out);
     hr_prof_end(ctx, PROF_PRE, st);
     HR_LAUNCHED(ctx);
     return HREBSD_OK;
@@ -196,24 +338,21 @@ extern "C" int hrebsd_background_batch(hrebsd_ctx *ctx, const float *in, int n, 
     int e = hr_set_device(ctx);
     if (e) return e;
     const size_t total = (size_t)n * H * W, plane = (size_t)H * W;
-    void *t0, *t1, *t2;
-    if ((e = hr_ws(ctx, WS_F0, total * 4, &t0)) || (e = hr_ws(ctx, WS_F1, total * 4, &t1)) ||
-        (e = hr_ws(ctx, WS_F2, total * 4, &t2)))
-        return e;
     cudaStream_t st = hr_stream(stream);
+    void *t0 = nullptr;
+    if (sigma_dyn > 0.0f && (e = hr_ws(ctx, WS_F0, total * 4, &t0))) return e;
+    float *x = (float *)t0;
     hr_prof_begin(ctx, st);
-    const float *cur = in;
-    if (static_bg) {
-        div_kernel<<<grid_of(ctx, total), 256, 0, st>>>(in, static_bg, (float *)t2, total, plane, 1);
+    if (sigma_dyn > 0.0f) {   // out may be in: the y pass reads each of its pixels just before it writes it
+        e = static_bg ? launch_pass<0, true, POST_NONE>(ctx, in, nullptr, static_bg, x, n, H, W, f, st)
+                      : launch_pass<0, false, POST_NONE>(ctx, in, nullptr, nullptr, x, n, H, W, f, st);
+        if (e) return e;
+        if ((e = launch_pass<1, false, POST_DIV>(ctx, x, in, static_bg, out, n, H, W, f, st))) return e;
+    } else if (static_bg) {
+        div_kernel<<<grid_of(ctx, total), 256, 0, st>>>(in, static_bg, out, total, plane);
         HR_LAUNCHED(ctx);
-        cur = (const float *)t2;
-    }
-    if (sigma_dyn > 0.0f) {
-        if ((e = blur_into(ctx, cur, (float *)t0, (float *)t1, n, H, W, f, st))) return e;
-        div_kernel<<<grid_of(ctx, total), 256, 0, st>>>(cur, (const float *)t1, out, total, plane, 0);
-        HR_LAUNCHED(ctx);
-    } else if (cur != out) {
-        HR_CHECK(cudaMemcpyAsync(out, cur, total * 4, cudaMemcpyDeviceToDevice, st));
+    } else if (in != out) {
+        HR_CHECK(cudaMemcpyAsync(out, in, total * 4, cudaMemcpyDeviceToDevice, st));
     }
     hr_prof_end(ctx, PROF_PRE, st);
     return HREBSD_OK;
