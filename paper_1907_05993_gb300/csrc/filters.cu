@@ -47,8 +47,9 @@ __device__ __forceinline__ float guarded_div(float a, float d) { return fabsf(d)
 // (pair, run) computes RUN consecutive outputs of its two lines: the window of RUN inputs sits in
 // registers (input j in slot j mod RUN, so nothing moves), a tap is one shared-memory load and RUN packed
 // FMAs.  Every output sums its taps in the order k = -r .. r, as one thread per output would.  Bound by
-// the FP32 FMAs from radius ~20 up (2r + 1 per pixel), by HBM below.  1000 patterns of 256 x 256, both
-// directions, radius 60 / 36 / 3: MEAS_BLUR.
+// the FP32 FMAs from radius ~20 up (2r + 1 per pixel), by HBM below.  1000 patterns of 256 x 256:
+// radius 3 101 us each direction (one thread per output and tap: 350), radius 60 373 us along x and 341
+// along y (was 2,900 each), the whole dynamic correction (radius 36) 730 us (was 4,000).
 //
 // The passes carry the element-wise steps around them, so that no intermediate image is written for
 // them: PRE divides the input by the background bg as it is loaded; POST divides the input of the
@@ -76,25 +77,40 @@ __global__ void __launch_bounds__(256, 3) blur_pass_kernel(BlurArgs a, const __g
     const int n_out = min(a.seg, len - s0), n_in = a.seg + 2 * r;
     const float *img = a.in + (AXIS ? blockIdx.y * plane : 0);
     float *sm = reinterpret_cast<float *>(blur_smem);
-    auto put = [&](int line, int j, float v) { sm[2 * ((line >> 1) * a.stride + j) + (line & 1)] = v; };
+    auto slot = [&](int line, int j) { return sm + 2 * ((line >> 1) * a.stride + j) + (line & 1); };
+    // asynchronous copies: every load of the tile is in flight at once
+    auto copy = [&](float *dst, const float *src) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                     : "memory");
+    };
     if (AXIS) {   // lanes on columns: coalesced loads, conflict-free stores
         const int line = threadIdx.x & 31, x = (int)l0 + line;
         if (x < W)
 #pragma unroll 4
             for (int j = threadIdx.x >> 5; j < n_in; j += (int)blockDim.x >> 5)
-                put(line, j, __ldg(img + (size_t)min(max(s0 - r + j, 0), H - 1) * W + x));
+                copy(slot(line, j), img + (size_t)min(max(s0 - r + j, 0), H - 1) * W + x);
     } else {
         for (int line = threadIdx.x >> 5; line < LINES; line += (int)blockDim.x >> 5) {
             const long long row = l0 + line;
             if (row >= a.lines) break;
-            const float *p = img + row * W, *bg = PRE ? a.bg + (size_t)(row % H) * W : nullptr;
+            const float *p = img + row * W;
 #pragma unroll 4
-            for (int j = threadIdx.x & 31; j < n_in; j += 32) {
-                const int x = min(max(s0 - r + j, 0), W - 1);
-                put(line, j, PRE ? guarded_div(__ldg(p + x), __ldg(bg + x)) : __ldg(p + x));
-            }
+            for (int j = threadIdx.x & 31; j < n_in; j += 32)
+                copy(slot(line, j), p + min(max(s0 - r + j, 0), W - 1));
         }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (PRE)   // every thread divides what it copied
+        for (int line = threadIdx.x >> 5; line < LINES; line += (int)blockDim.x >> 5) {
+            const long long row = l0 + line;
+            if (row >= a.lines) break;
+            const float *bg = a.bg + (size_t)(row % H) * W;
+#pragma unroll 4
+            for (int j = threadIdx.x & 31; j < n_in; j += 32) {
+                float *p = slot(line, j);
+                *p = guarded_div(*p, __ldg(bg + min(max(s0 - r + j, 0), W - 1)));
+            }
+        }
     __syncthreads();
     // an odd number of runs leaves half a warp over: it repeats the last run and stores nothing
     const int pr = threadIdx.x % PAIRS, o0 = min((int)threadIdx.x / PAIRS * RUN, a.seg - RUN);
@@ -125,27 +141,36 @@ __global__ void __launch_bounds__(256, 3) blur_pass_kernel(BlurArgs a, const __g
         if (k + u < 2 * r) win[u] = q[k + u + RUN];
     }
     if (AXIS) {
-        const int x = (int)l0 + 2 * pr;
+        const int x = (int)l0 + 2 * pr, rows = live && x < W ? n_out - o0 : 0;   // this thread's outputs
         const bool two = x + 1 < W;
+        const size_t p0 = (size_t)(s0 + o0) * W + x, at0 = blockIdx.y * plane + p0;
+        if (POST != POST_NONE) {   // all loads of the run before any use (src may be out: read here, written below)
+            float2 c[RUN];
+#pragma unroll
+            for (int i = 0; i < RUN; ++i)
+                c[i] = i < rows ? make_float2(a.src[at0 + (size_t)i * W], two ? a.src[at0 + (size_t)i * W + 1] : 0.0f)
+                                : make_float2(0.0f, 0.0f);
+            if (POST == POST_DIV && a.bg)
+#pragma unroll
+                for (int i = 0; i < RUN; ++i)
+                    if (i < rows) {
+                        c[i].x = guarded_div(c[i].x, __ldg(a.bg + p0 + (size_t)i * W));
+                        if (two) c[i].y = guarded_div(c[i].y, __ldg(a.bg + p0 + (size_t)i * W + 1));
+                    }
+#pragma unroll
+            for (int i = 0; i < RUN; ++i)
+                acc[i] = POST == POST_DIV ? make_float2(guarded_div(c[i].x, acc[i].x), guarded_div(c[i].y, acc[i].y))
+                                          : make_float2(c[i].x - acc[i].x, c[i].y - acc[i].y);
+        }
 #pragma unroll
         for (int i = 0; i < RUN; ++i) {
-            if (o0 + i >= n_out || x >= W || !live) break;
-            const size_t p = (size_t)(s0 + o0 + i) * W + x, at = blockIdx.y * plane + p;
-            float2 v = acc[i];
-            if (POST != POST_NONE) {
-                float2 c = make_float2(a.src[at], two ? a.src[at + 1] : 0.0f);   // src may be out
-                if (POST == POST_DIV && a.bg) {
-                    c.x = guarded_div(c.x, __ldg(a.bg + p));
-                    if (two) c.y = guarded_div(c.y, __ldg(a.bg + p + 1));
-                }
-                v = POST == POST_DIV ? make_float2(guarded_div(c.x, v.x), guarded_div(c.y, v.y))
-                                     : make_float2(c.x - v.x, c.y - v.y);
-            }
+            if (i >= rows) break;
+            float *o = a.out + at0 + (size_t)i * W;
             if (a.vec) {
-                *reinterpret_cast<float2 *>(a.out + at) = v;
+                *reinterpret_cast<float2 *>(o) = acc[i];
             } else {
-                a.out[at] = v.x;
-                if (two) a.out[at + 1] = v.y;
+                o[0] = acc[i].x;
+                if (two) o[1] = acc[i].y;
             }
         }
     } else {   // through shared memory, so that rows are written whole
@@ -170,8 +195,19 @@ __global__ void div_kernel(const float *a, const float *d, float *out, size_t to
         out[i] = guarded_div(a[i], d[i % plane]);
 }
 
-// Mean over the n images: 32 pixels x 8 groups of images per CTA, summed in FP64, the groups' sums added in
-// order.  Bound by the FP64 additions (2 per clock and SM): 1000 patterns of 256 x 256 in MEAS_MEAN.
+// s + v exactly as s + e (Knuth's two-sum)
+__device__ __forceinline__ void two_sum(float &s, float v, float &e)
+{
+    const float t = s + v, b = t - s;
+    e = (s - (t - b)) + (v - b);
+    s = t;
+}
+
+// Mean over the n images: 32 pixels x 8 groups of images per CTA.  FP64 additions and conversions would
+// bound it (1000 patterns of 256 x 256: 289 us with one thread per pixel, 261 us with this split), so a
+// group sums in three FP32 parts with exact carries, which hold more bits than one FP64 sum, and only the
+// parts and the groups' sums are added in FP64 (49 us; the read alone takes 39).  Sums that leave the range of FP32 (or are not
+// finite) are repeated in FP64.
 __global__ void __launch_bounds__(256) mean_pattern_kernel(const float *__restrict__ in, int n, size_t plane, float *out)
 {
     __shared__ double part[8][32];
@@ -180,16 +216,26 @@ __global__ void __launch_bounds__(256) mean_pattern_kernel(const float *__restri
     double s = 0.0;
     if (p < plane) {
         const float *q = in + p;
+        float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, e;
+        auto add = [&](float v) {
+            two_sum(s0, v, e);
+            two_sum(s1, e, e);
+            s2 += e;
+        };
         int i = grp;
-        for (; i + 24 < n; i += 32) {
-            const float v0 = __ldg(q + (size_t)i * plane), v1 = __ldg(q + (size_t)(i + 8) * plane);
-            const float v2 = __ldg(q + (size_t)(i + 16) * plane), v3 = __ldg(q + (size_t)(i + 24) * plane);
-            s += v0;
-            s += v1;
-            s += v2;
-            s += v3;
+        for (; i + 56 < n; i += 64) {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = __ldg(q + (size_t)(i + 8 * j) * plane);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) add(v[j]);
         }
-        for (; i < n; i += 8) s += __ldg(q + (size_t)i * plane);
+        for (; i < n; i += 8) add(__ldg(q + (size_t)i * plane));
+        s = (double)s0 + ((double)s1 + (double)s2);
+        if (!isfinite(s)) {
+            s = 0.0;
+            for (i = grp; i < n; i += 8) s += __ldg(q + (size_t)i * plane);
+        }
     }
     part[grp][lane] = s;
     __syncthreads();
