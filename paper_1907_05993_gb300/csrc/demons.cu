@@ -115,15 +115,29 @@ __device__ __forceinline__ void warp_cell_f(float q, float u, float m2, int &i, 
     i = (int)xc;
 }
 
-// warp_cell_f with the cell index returned as a float (integer-valued, exact): the texture
-// coordinate of the cell's four-texel gather.  Same cell and weight.
-__device__ __forceinline__ void warp_cell_ff(float q, float u, float m2, float &xc, float &f)
+// Both axes of warp_cell_f in packed FP32x2 steps: the pixel q - u, cells c (integer-valued floats) and
+// weights f, m2 the largest cells.  With n' = ceil(u) = -floor(-u), a - b as fma(b, -1, a): the same
+// rounding steps, so the same cell and weight.
+__device__ __forceinline__ void warp_cell2(float2 q, float2 u, float2 m2, float2 &c, float2 &f)
 {
-    const float n = floorf(-u);
-    const float fr = -u - n;
-    const float x = q + n;
-    xc = fminf(fmaxf(x, 0.0f), m2);
-    f = __saturatef(fr + (x - xc));
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    const float2 n = make_float2(ceilf(u.x), ceilf(u.y));
+    const float2 fr = __ffma2_rn(u, m1, n);
+    const float2 x = __ffma2_rn(n, m1, q);
+    c = make_float2(fminf(fmaxf(x.x, 0.0f), m2.x), fminf(fmaxf(x.y, 0.0f), m2.y));
+    const float2 o = __ffma2_rn(c, m1, x);
+    f = make_float2(__saturatef(fr.x + o.x), __saturatef(fr.y + o.y));
+}
+
+// The step length of Eq. 1, d / den, 0 where den <= 1e-9: a product with the approximate reciprocal (what
+// __fdividef does, without its extra scaling for divisors above 2^126) and a select, so that no branch
+// splits the pixels of a run.
+__device__ __forceinline__ float force_quot(float d, float den)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(den));
+    const float t = d * r;
+    return den > 1e-9f ? t : 0.0f;
 }
 
 // Bilinear sample of M at the point (qx - ux, qy - uy), clamped to the image;
@@ -414,7 +428,7 @@ __global__ void __launch_bounds__(kIterThreads, 2) demons_iter_kernel(IterArgs a
             const float mw = warp_sample(M, h, w, qx, qy, u.x, u.y);
             const float d = mw - fc[0];
             const float den = fmaf(gx, gx, fmaf(gy, gy, a.alpha2 * d * d));
-            const float t = den > 1e-9f ? __fdividef(d, den) : 0.0f;
+            const float t = force_quot(d, den);
             du = make_float2(t * gx, t * gy);
             const bool in_T = r >= RAD && r < RAD + TY && c >= RAD && c < RAD + TX && vy < h && vx < w;
             d2 = in_T ? d * d : 0.0f;
@@ -759,7 +773,7 @@ __global__ void __launch_bounds__(NT_, MINB) demons_iter_tma_kernel(const __grid
                 for (int j = 0; j < 2; ++j) {
                     const int r = r0 + i + j;
                     const float dj = j ? d.y : d.x, denj = j ? den.y : den.x;
-                    const float t = denj > 1e-9f ? __fdividef(dj, denj) : 0.0f;
+                    const float t = force_quot(dj, denj);
                     const float2 g = j ? make_float2(gx.y, gy.y) : make_float2(gx.x, gy.x);
                     if (L::BH % FR == 0 || r < L::BH) sD[r * L::DST + c] = __fmul2_rn(make_float2(t, t), g);
                     if (colT && (unsigned)(r - RAD) < (unsigned)rows_in) ssd = fmaf(dj, dj, ssd);
@@ -1619,7 +1633,8 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
         const bool use_level = var == kLevelVariant && level_ok(rad, h, w) && cap >= 1;
         if (var == kLevelVariant && !use_level) var = kStripVariant;
         const bool sweep_v = var == kStripVariant || var == kLoopVariant;
-        const bool use_strip = sweep_v && strip_ok(rad, w) && !ctx->no_tma;
+        // (the row sweep forms pixel offsets in FP32: levels below 2^24 pixels)
+        const bool use_strip = sweep_v && strip_ok(rad, w) && (long long)h * w < (1 << 24) && !ctx->no_tma;
         if (sweep_v && !use_strip) var = 4;   // the row sweep does not cover this level: 64x64 tiles
         // the whole level after iteration 0 in one launch (needs the stop rule's history: cap > 1):
         // shape 6, or shape 5 when every pair has a CTA of its own, so that no pair waits for another

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(NT, 2) demons_level_kernel(LevelArgs a)
                     const float gx = sx * fmaf(fl, -1.0f, frt), gy = sy * fmaf(fup, -1.0f, fdn);
                     const float d = fmaf(fc, -1.0f, mw);
                     const float den = fmaf(gx, gx, fmaf(gy, gy, (al2 * d) * d));
-                    const float tt = den > 1e-9f ? __fdividef(d, den) : 0.0f;
+                    const float tt = force_quot(d, den);
                     A[swz(y, x)] = make_float2(tt * gx, tt * gy);
                     ssd = fmaf(d, d, ssd);
                 }

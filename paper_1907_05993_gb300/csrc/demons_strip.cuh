@@ -27,7 +27,7 @@
 // last DX row is pushed again.  A window of 2r + 1 = R rows keeps row y in
 // slot y mod R, so its slots are compile-time indices in the unrolled row loop
 // and nothing moves between registers.  The s and test-image rows of step
-// k + 2 are requested by bulk copies (one per row, issued by 16 lanes of one
+// k + 2 are requested by bulk copies (one per row, an equal share by each
 // warp, completion on an mbarrier that every thread waits on with a bounded
 // wait) as soon as step k's barrier shows its buffer consumed.
 namespace strip {
@@ -44,8 +44,8 @@ struct Geo {
     static constexpr int HST = NT + 10;                 // float2 stride of halo rows (odd 16-byte slots)
     static constexpr int XST = NT + 10;                 // float2 stride of RX / DX rows (the same)
     static constexpr int FR_ = R + 2;                   // test-image rows of a step
-    static constexpr int FST = NT + 4;                  // float stride of test-image rows (odd 16-byte slots)
-    static_assert((HST / 2) % 2 == 1 && (XST / 2) % 2 == 1 && (FST / 4) % 2 == 1, "odd numbers of 16-byte slots");
+    static constexpr int FST = NT;                      // float stride of test-image rows (read along rows only)
+    static_assert((HST / 2) % 2 == 1 && (XST / 2) % 2 == 1, "odd numbers of 16-byte slots");
     static_assert((HST / 2) % 8 == 5 && (XST / 2) % 8 == 5, "the x-pass lane map below is conflict-free for 5 mod 8");
     static constexpr size_t S_OFF = 0;                                   // s rows [2][R][HST] float2
     static constexpr size_t F_OFF = S_OFF + (size_t)2 * R * HST * 8;     // test rows [2][FR_][FST] float
@@ -53,32 +53,42 @@ struct Geo {
     static constexpr size_t X_OFF = D_OFF + (size_t)2 * R * HST * 8;     // RX rows [R][XST] float2
     static constexpr size_t Y_OFF = X_OFF + (size_t)R * XST * 8;         // DX rows [R][XST] float2
     static constexpr size_t BYTES = Y_OFF + (size_t)R * XST * 8;
-    static constexpr uint32_t S_BYTES = (uint32_t)R * NT * 8;            // bytes of a step's s rows
-    static constexpr uint32_t F_BYTES = (uint32_t)FR_ * NT * 4;          // ... and test-image rows
     static_assert(S_OFF % 16 == 0 && F_OFF % 16 == 0 && X_OFF % 16 == 0 && D_OFF % 16 == 0 && Y_OFF % 16 == 0,
                   "16-byte aligned regions");
 };
 
 // The bulk copies of step k of a pair into one buffer: s rows clamp(R k + i) (i < R) of the pair's
 // plane sp (when copy_s) and test-image rows clamp(R k - r - 1 + i) (i < R + 2) of its plane fp, whole
-// rows.  Called by every lane of one warp: lane 0 announces the bytes, then lanes 0 .. R - 1 copy the
-// s rows and lanes R .. 2R + 1 the test rows.
+// rows: one copy per s row (their rows are padded in shared memory), one copy for the test rows where
+// none is clamped, else one per row.  Every warp calls it (whole) and issues an equal share: a bulk copy
+// takes its operands from uniform registers, so the copies of one warp are issued one after another
+// (~20 instructions each), and a single issuing warp held up the others at every step's barrier.  The
+// warp's first lane announces the share's bytes.
 template <int RAD, int NT>
 __device__ __forceinline__ void issue_step(bool copy_s, const float2 *sp, const float *fp, int h, int k, float2 *sS,
-                                           float *sF, uint64_t *bar, int lane)
+                                           float *sF, uint64_t *bar, int warp, int lane)
 {
     using G = Geo<RAD, NT>;
-    if (lane == 0) hr_tma::mbar_arrive_expect_tx(bar, (copy_s ? G::S_BYTES : 0u) + G::F_BYTES);
-    __syncwarp();
-    if (lane < R) {
-        if (copy_s) {
-            hr_tma::fence_proxy_async();   // the buffer's previous contents were read by the generic proxy
-            hr_tma::load_bulk(sS + lane * G::HST + G::HO, sp + (size_t)min(R * k + lane, h - 1) * NT, NT * 8, bar);
+    constexpr int NWARP = NT / 32, SHARE = (R + 1) / NWARP;
+    static_assert((R + 1) % NWARP == 0, "equal shares of the R s rows and the test rows");
+    if (lane != 0) return;
+    const bool has_f = warp == NWARP - 1;   // its last item is the test rows
+    hr_tma::mbar_arrive_expect_tx(bar, (copy_s ? (has_f ? SHARE - 1 : SHARE) * NT * 8 : 0) + (has_f ? G::FR_ * NT * 4 : 0));
+    hr_tma::fence_proxy_async();   // the buffer's previous contents were read by the generic proxy
+    if (copy_s)
+#pragma unroll
+        for (int j = 0; j < SHARE; ++j) {
+            const int row = warp * SHARE + j;
+            if (j + 1 < SHARE || !has_f)
+                hr_tma::load_bulk(sS + row * G::HST + G::HO, sp + (size_t)min(R * k + row, h - 1) * NT, NT * 8, bar);
         }
-    } else if (lane < R + G::FR_) {
-        const int i = lane - R;
-        hr_tma::fence_proxy_async();
-        hr_tma::load_bulk(sF + i * G::FST, fp + (size_t)min(max(R * k - RAD - 1 + i, 0), h - 1) * NT, NT * 4, bar);
+    if (has_f) {
+        const int y0 = R * k - RAD - 1;
+        if (y0 >= 0 && y0 + G::FR_ <= h)
+            hr_tma::load_bulk(sF, fp + (size_t)y0 * NT, G::FR_ * NT * 4, bar);
+        else
+            for (int i = 0; i < G::FR_; ++i)
+                hr_tma::load_bulk(sF + i * NT, fp + (size_t)min(max(y0 + i, 0), h - 1) * NT, NT * 4, bar);
     }
 }
 
@@ -140,7 +150,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
     __shared__ int s_next;   // LOOP: the pair's next iteration, or -1 once the stop rule ended it
     __shared__ int s_item;   // LOOP: the item taken from the counter
 
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, lane = t & 31, warp = __shfl_sync(0xffffffffu, t >> 5, 0);   // (warp uniform)
     constexpr int NWARP = NT / 32;
     // the Gaussian taps are symmetric (t[j] = t[2r - j]): half of them in registers
     float2 tfh[RAD + 1], tuh[RAD + 1];
@@ -161,8 +171,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
         if (a.px_count) atomicAdd(a.px_count, (unsigned long long)n_active * a.h * a.w);
     }
     if (t == 0) {
-        hr_tma::mbar_init(&bar[0], 1);
-        hr_tma::mbar_init(&bar[1], 1);
+        hr_tma::mbar_init(&bar[0], NWARP);
+        hr_tma::mbar_init(&bar[1], NWARP);
         hr_tma::fence_mbar_init();
     }
     __syncthreads();
@@ -217,11 +227,11 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
         item = s_item;
     }
     uint32_t g = 0;   // steps of this CTA so far: step g uses buffer g & 1, phase parity (g >> 1) & 1
-    if (warp == 0 && item < n_active) {
+    if (item < n_active) {
         const int p0 = a.active[item];
-        issue_step<RAD, NT>(IN_S, src_of(p0, K_FIRST), fsrc_of(p0), h, 0, sS0, sF0, &bar[0], lane);
+        issue_step<RAD, NT>(IN_S, src_of(p0, K_FIRST), fsrc_of(p0), h, 0, sS0, sF0, &bar[0], warp, lane);
         issue_step<RAD, NT>(IN_S, src_of(p0, K_FIRST), fsrc_of(p0), h, 1, sS0 + R * G::HST, sF0 + G::FR_ * G::FST,
-                            &bar[1], lane);
+                            &bar[1], warp, lane);
     }
     while (item < n_active) {
         const int pair = a.active[item];
@@ -319,87 +329,88 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
                     }
                     ucur[i] = u;
                 }
-                float mA[R], mB[R], mC[R], mD[R], fxv[R], fyv[R];
+                // the cell's pixels (x0, y0 + 1), (x0 + 1, y0 + 1), (x0 + 1, y0), (x0, y0), in the order in
+                // which a texture gather returns them
+                float4 m[R];
+                float fxv[R], fyv[R];
+                float2 q = make_float2(tf_, yk);   // the pixel's coordinates (exact integers)
 #pragma unroll
                 for (int i = 0; i < R; ++i) {
                     const int yu = R * k + i - RAD;
-                    // row coordinate as a float (exact integers); rows outside: any valid cell
-                    const float yc = IN ? yk + (float)i : (float)min(max(yu, 0), h - 1);
+                    if (!IN) q.y = (float)min(max(yu, 0), h - 1);   // rows outside: any valid cell
+                    float2 c, f;
+                    warp_cell2(q, ucur[i], make_float2(mx2, my2), c, f);
+                    if (IN) q = __fadd2_rn(q, make_float2(0.0f, 1.0f));
+                    fxv[i] = f.x;
+                    fyv[i] = f.y;
                     if constexpr (TEX) {
-                        // one gather returns (x0, y0 + 1), (x0 + 1, y0 + 1), (x0 + 1, y0), (x0, y0)
-                        float xc, ycl;
-                        warp_cell_ff(tf_, ucur[i].x, mx2, xc, fxv[i]);
-                        warp_cell_ff(yc, ucur[i].y, my2, ycl, fyv[i]);
-                        const float4 q = tex2Dgather<float4>(a.mtex, xc + 1.0f, ycl + yt, 0);
-                        mA[i] = q.w;
-                        mB[i] = q.z;
-                        mC[i] = q.x;
-                        mD[i] = q.y;
-                    } else {
-                        int x0, y0;
-                        warp_cell_f(tf_, ucur[i].x, mx2, x0, fxv[i]);
-                        warp_cell_f(yc, ucur[i].y, my2, y0, fyv[i]);
-                        const float *p = M + y0 * NT + x0;
-                        mA[i] = __ldg(p);
-                        mB[i] = __ldg(p + 1);
-                        mC[i] = __ldg(p + NT);
-                        mD[i] = __ldg(p + NT + 1);
+                        const float2 g = __fadd2_rn(c, make_float2(1.0f, yt));
+                        m[i] = tex2Dgather<float4>(a.mtex, g.x, g.y, 0);
+                    } else {   // (level sizes below 2^24 pixels: exact in FP32, as the coordinates are)
+                        const float *p = M + (int)fmaf(c.y, (float)NT, c.x);
+                        m[i] = make_float4(__ldg(p + NT), __ldg(p + NT + 1), __ldg(p + 1), __ldg(p));
                     }
                 }
-                // the force of one row (scalar) ...
-                auto force1 = [&](int i, int yu) {
-                    // test image rows yu - 1 .. yu + 1 are staged rows i .. i + 2
-                    const float *fr_ = sF + i * G::FST;
-                    const float fc = fr_[G::FST + t], fup = fr_[t], fdn = fr_[2 * G::FST + t];
-                    const float fl = fr_[G::FST + tl], frt = fr_[G::FST + tr];
-                    const float sy = (!IN && (yu == 0 || yu == h - 1)) ? 1.0f : 0.5f;
+                // The force of one row (scalar; test image rows yu - 1 .. yu + 1 are staged rows i .. i + 2) ...
+                auto force1 = [&](int i, float fup, float fc, float fdn, float sy) {
+                    const float *fr_ = sF + (i + 1) * G::FST;
+                    const float fl = fr_[tl], frt = fr_[tr];
                     const float fx = fxv[i], fy = fyv[i];
                     const float omx = fmaf(fx, -1.0f, 1.0f), omy = fmaf(fy, -1.0f, 1.0f);
-                    const float top = fmaf(fx, mB[i], omx * mA[i]), bot = fmaf(fx, mD[i], omx * mC[i]);
+                    const float top = fmaf(fx, m[i].z, omx * m[i].w), bot = fmaf(fx, m[i].y, omx * m[i].x);
                     const float mw = fmaf(fy, bot, omy * top);
                     const float gx = sx * fmaf(fl, -1.0f, frt), gy = sy * fmaf(fup, -1.0f, fdn);
                     const float d = fmaf(fc, -1.0f, mw);
-                    const float den = fmaf(gx, gx, fmaf(gy, gy, (al2 * d) * d));
-                    const float tt = den > 1e-9f ? __fdividef(d, den) : 0.0f;
+                    const float tt = force_quot(d, fmaf(gx, gx, fmaf(gy, gy, (al2 * d) * d)));
                     sD[i * G::HST + G::HO + t] = make_float2(tt * gx, tt * gy);
                     ssd = fmaf(d, d, ssd);
                 };
-                // ... and of rows i, i + 1 of an interior step in packed FP32x2 arithmetic (every
-                // rounding step that of force1: a - b as fma(b, -1, a), products and fmas in order)
-                auto force2 = [&](int i) {
-                    const float *fr_ = sF + i * G::FST;
-                    const float f0 = fr_[t], f1 = fr_[G::FST + t], f2 = fr_[2 * G::FST + t], f3 = fr_[3 * G::FST + t];
-                    const float2 fl = make_float2(fr_[G::FST + tl], fr_[2 * G::FST + tl]);
-                    const float2 frt = make_float2(fr_[G::FST + tr], fr_[2 * G::FST + tr]);
+                // ... and of rows i, i + 1 of an interior step, in packed FP32x2 arithmetic where the
+                // operands pair up without moves (every rounding step that of force1: a - b as
+                // fma(b, -1, a), products and fmas in order; the gathered pixels come four to a register
+                // group, so their interpolation along x is scalar)
+                auto force2 = [&](int i, float f0, float f1, float f2, float f3) {
+                    const float *fr_ = sF + (i + 1) * G::FST;
+                    const float2 fl = make_float2(fr_[tl], fr_[G::FST + tl]);
+                    const float2 frt = make_float2(fr_[tr], fr_[G::FST + tr]);
                     const float2 n1 = make_float2(-1.0f, -1.0f), one = make_float2(1.0f, 1.0f);
                     const float2 fx = make_float2(fxv[i], fxv[i + 1]), fy = make_float2(fyv[i], fyv[i + 1]);
                     const float2 omx = __ffma2_rn(fx, n1, one), omy = __ffma2_rn(fy, n1, one);
-                    const float2 top = __ffma2_rn(fx, make_float2(mB[i], mB[i + 1]),
-                                                  __fmul2_rn(omx, make_float2(mA[i], mA[i + 1])));
-                    const float2 bot = __ffma2_rn(fx, make_float2(mD[i], mD[i + 1]),
-                                                  __fmul2_rn(omx, make_float2(mC[i], mC[i + 1])));
+                    const float2 top = make_float2(fmaf(fx.x, m[i].z, omx.x * m[i].w),
+                                                   fmaf(fx.y, m[i + 1].z, omx.y * m[i + 1].w));
+                    const float2 bot = make_float2(fmaf(fx.x, m[i].y, omx.x * m[i].x),
+                                                   fmaf(fx.y, m[i + 1].y, omx.y * m[i + 1].x));
                     const float2 mw = __ffma2_rn(fy, bot, __fmul2_rn(omy, top));
                     const float2 gx = __fmul2_rn(make_float2(sx, sx), __ffma2_rn(fl, n1, frt));
                     const float2 gy = __fmul2_rn(make_float2(0.5f, 0.5f), __ffma2_rn(make_float2(f0, f1), n1, make_float2(f2, f3)));
-                    const float2 d = __ffma2_rn(make_float2(f1, f2), n1, mw);
+                    const float2 d = make_float2(fmaf(f1, -1.0f, mw.x), fmaf(f2, -1.0f, mw.y));
                     const float2 a2 = make_float2(al2, al2);
                     const float2 den = __ffma2_rn(gx, gx, __ffma2_rn(gy, gy, __fmul2_rn(__fmul2_rn(a2, d), d)));
-                    const float t0 = den.x > 1e-9f ? __fdividef(d.x, den.x) : 0.0f;
-                    const float t1 = den.y > 1e-9f ? __fdividef(d.y, den.y) : 0.0f;
+                    const float t0 = force_quot(d.x, den.x), t1 = force_quot(d.y, den.y);
                     sD[i * G::HST + G::HO + t] = make_float2(t0 * gx.x, t0 * gy.x);
                     sD[(i + 1) * G::HST + G::HO + t] = make_float2(t1 * gx.y, t1 * gy.y);
                     ssd = fmaf(d.x, d.x, ssd);
                     ssd = fmaf(d.y, d.y, ssd);
                 };
+                // the column's staged rows are read once, two rows ahead
+                float fa = sF[t], fb = sF[G::FST + t];
                 if (IN) {
 #pragma unroll
-                    for (int i = 0; i + 1 < R; i += 2) force2(i);
-                    force1(R - 1, R * k - RAD + R - 1);
+                    for (int i = 0; i + 1 < R; i += 2) {
+                        const float f2 = sF[(i + 2) * G::FST + t], f3 = sF[(i + 3) * G::FST + t];
+                        force2(i, fa, fb, f2, f3);
+                        fa = f2;
+                        fb = f3;
+                    }
+                    force1(R - 1, fa, fb, sF[(R + 1) * G::FST + t], 0.5f);
                 } else {
 #pragma unroll
                     for (int i = 0; i < R; ++i) {
                         const int yu = R * k + i - RAD;
-                        if (yu >= 0 && yu < h) force1(i, yu);
+                        const float fn = sF[(i + 2) * G::FST + t];
+                        if (yu >= 0 && yu < h) force1(i, fa, fb, fn, (yu == 0 || yu == h - 1) ? 1.0f : 0.5f);
+                        fa = fb;
+                        fb = fn;
                     }
                 }
             };
@@ -415,13 +426,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
                 }
                 return;
             }
-            if (warp == 0) {   // step k + 2 into the buffer just consumed
-                if (k + 2 < nsteps)
-                    issue_step<RAD, NT>(IN_S, sp, fp, h, k + 2, sS, sF, &bar[b], lane);
-                else if (!LOOP && next_pair >= 0)
-                    issue_step<RAD, NT>(IN_S, src_of(next_pair, K_FIRST), fsrc_of(next_pair), h, k + 2 - nsteps, sS,
-                                        sF, &bar[b], lane);
-            }
+            // step k + 2 into the buffer just consumed
+            if (k + 2 < nsteps)
+                issue_step<RAD, NT>(IN_S, sp, fp, h, k + 2, sS, sF, &bar[b], warp, lane);
+            else if (!LOOP && next_pair >= 0)
+                issue_step<RAD, NT>(IN_S, src_of(next_pair, K_FIRST), fsrc_of(next_pair), h, k + 2 - nsteps, sS, sF,
+                                    &bar[b], warp, lane);
+            __syncwarp();
             // ---- x pass of G_u on the du rows that exist -> DX (the warp's own columns; the edge
             // warps first fill the halo columns with the edge values)
             fill_halo(sD);
@@ -471,20 +482,20 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
         const int nk = s_next;
         if (nk < 0) {   // the pair is done: the next item's first two steps
             next_item = s_item;
-            if (warp == 0 && next_item < n_active) {
+            if (next_item < n_active) {
                 const int np = a.active[next_item];
                 issue_step<RAD, NT>(true, src_of(np, K_FIRST), fsrc_of(np), h, 0, sS0 + (g & 1) * R * G::HST,
-                                    sF0 + (g & 1) * G::FR_ * G::FST, &bar[g & 1], lane);
+                                    sF0 + (g & 1) * G::FR_ * G::FST, &bar[g & 1], warp, lane);
                 issue_step<RAD, NT>(true, src_of(np, K_FIRST), fsrc_of(np), h, 1, sS0 + ((g + 1) & 1) * R * G::HST,
-                                    sF0 + ((g + 1) & 1) * G::FR_ * G::FST, &bar[(g + 1) & 1], lane);
+                                    sF0 + ((g + 1) & 1) * G::FR_ * G::FST, &bar[(g + 1) & 1], warp, lane);
             }
             break;
         }
-        if (warp == 0) {   // the pair's next iteration: its first two steps
+        {   // the pair's next iteration: its first two steps
             issue_step<RAD, NT>(true, src_of(pair, nk), fp, h, 0, sS0 + (g & 1) * R * G::HST,
-                                sF0 + (g & 1) * G::FR_ * G::FST, &bar[g & 1], lane);
+                                sF0 + (g & 1) * G::FR_ * G::FST, &bar[g & 1], warp, lane);
             issue_step<RAD, NT>(true, src_of(pair, nk), fp, h, 1, sS0 + ((g + 1) & 1) * R * G::HST,
-                                sF0 + ((g + 1) & 1) * G::FR_ * G::FST, &bar[(g + 1) & 1], lane);
+                                sF0 + ((g + 1) & 1) * G::FR_ * G::FST, &bar[(g + 1) & 1], warp, lane);
         }
       }
         item = next_item;
