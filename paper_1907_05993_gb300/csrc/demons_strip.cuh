@@ -12,13 +12,13 @@
 //     cell's four pixels from a CUDA-array copy of the references, else four
 //     loads) are issued for all R rows before any of them is used, then the
 //     force of Eq. 1 (test-image rows staged in shared memory)  -> du rows;
-//   one CTA barrier (the du rows' x pass reads r columns of the neighbouring
-//     warps);
+//   each warp arrives on an mbarrier (the du rows' x pass reads r columns of the
+//     neighbouring warps) and runs the next step's x pass of G_f before it waits;
 //   x pass of G_u on the du rows, for the warp's own columns     -> DX rows;
-// and, at the start of the next step, per column: the y pass of G_u over a
-// rolling window of DX rows, plus u, gives s_{k+1} (lagging by 2r rows),
-// stored to HBM.  Everything but the du rows stays within a warp, so a step
-// has a single CTA barrier (du rows alternate between two buffers).
+//   per column, the y pass of G_u over a rolling window of DX rows, plus u, gives
+//     s_{k+1} (lagging by 2r rows), stored to HBM.
+// Everything but the du rows stays within a warp, so the warps meet once per
+// step (du rows alternate between two buffers).
 // The separable passes read each input once per output in the vertical
 // direction (register windows) and have no halo rows at all; the x passes
 // read r halo columns on each side, which hold the row's edge values
@@ -146,7 +146,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
     float2 *sRX = reinterpret_cast<float2 *>(smraw + G::X_OFF);
     float2 *sDX = reinterpret_cast<float2 *>(smraw + G::Y_OFF);
     __shared__ float red[NT / 32];
-    __shared__ __align__(8) uint64_t bar[2];
+    __shared__ __align__(8) uint64_t bar[2];   // a step's copies
+    __shared__ __align__(8) uint64_t dbar;     // a step's du rows: every warp arrives, then waits
     __shared__ int s_next;   // LOOP: the pair's next iteration, or -1 once the stop rule ended it
     __shared__ int s_item;   // LOOP: the item taken from the counter
 
@@ -173,6 +174,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
     if (t == 0) {
         hr_tma::mbar_init(&bar[0], NWARP);
         hr_tma::mbar_init(&bar[1], NWARP);
+        hr_tma::mbar_init(&dbar, NWARP);
         hr_tma::fence_mbar_init();
     }
     __syncthreads();
@@ -220,7 +222,22 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
     auto fsrc_of = [&](int pair) { return a.Ftest + (size_t)pair * plane; };
     constexpr int K_FIRST = LOOP ? 1 : 0;   // the iteration of an item's first sweep (LOOP: after k = 0)
 
+    // Step gg's rows (counted over the CTA's life): wait for its copies (bounded), then the x pass of
+    // G_f on its s rows -> RX, the warp's own columns (the edge warps first fill the halo columns of the
+    // rows with the edge values).  False when the copies did not arrive.
+    auto stage = [&](uint32_t gg) {
+        bool ok = hr_tma::mbar_wait(&bar[gg & 1], (gg >> 1) & 1u);
+        if (IN_S) {
+            float2 *sS = sS0 + (gg & 1) * R * G::HST;
+            fill_halo(sS);
+            if (xlane) run_x_halo<RAD>(sS + xi * G::HST, xc0, sRX + xi * G::XST + xc0, tf);
+            __syncwarp();
+        }
+        return ok;
+    };
+
     int item = blockIdx.x;
+    bool primed = false;   // the first step of the next sweep is staged
     if (LOOP) {
         if (t == 0) s_item = atomicAdd(c.work, 1);
         __syncthreads();
@@ -249,61 +266,13 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
         float2 *dst = dst_of(pair, kit);
         float2 rxw[R], dxw[R], ucur[R], uprev[RAD], last_dx = make_float2(0.0f, 0.0f);
         float ssd = 0.0f;
-        for (int k = 0; k <= nsteps; ++k) {
-            // ---- outputs of step k - 1: y pass of G_u over the DX window, s = u + G_u * du
-            // (DX rows of the warp's own columns, written by this warp before its __syncwarp).
-            // Interior steps (every row inside, none at an edge) run without the edge handling.
-            if (k > 0) {
-                const int kp = k - 1;
-                float2 *dk = dst + (ptrdiff_t)(R * kp - 2 * RAD) * NT + t;   // row yo for i = 0
-                auto outputs = [&](auto interior) {
-                    constexpr bool IN = decltype(interior)::value;
-#pragma unroll
-                    for (int i = 0; i < R; ++i) {
-                        const int yu = R * kp + i - RAD, yo = yu - RAD;   // du row entering, output row
-                        if (IN || yu >= 0) {
-                            const float2 v = (IN || yu < h) ? sDX[i * G::XST + t] : last_dx;
-                            if (!IN && yu < h) last_dx = v;
-                            dxw[(i + R - RAD) % R] = v;   // row yu in slot yu mod R
-                            if (!IN && yu == 0) {
-#pragma unroll
-                                for (int j = 0; j < R; ++j) dxw[j] = v;
-                            }
-                        }
-                        if (IN || (yo >= 0 && yo < h)) {
-                            // rows yo - r + j = yu - 2r + j sit in slots (i - 3r + j) mod R
-                            float2 acc = __fmul2_rn(tu[0], dxw[(i + 2 * R - 3 * RAD) % R]);
-#pragma unroll
-                            for (int j = 1; j < R; ++j) acc = ffma2(tu[j], dxw[(i + 2 * R - 3 * RAD + j) % R], acc);
-                            const float2 uo = i >= RAD ? ucur[i - RAD] : uprev[i];
-                            dk[i * NT] = __fadd2_rn(uo, acc);   // row yo
-                        }
-                    }
-                };
-                if (interior_step(kp)) outputs(std::true_type());
-                else outputs(std::false_type());
-#pragma unroll
-                for (int i = 0; i < RAD; ++i) uprev[i] = ucur[R - RAD + i];
-            }
-            if (k == nsteps) {
-                // LOOP: the next iteration's bulk copies read these rows of s_{k+1} (async proxy)
-                if (LOOP) asm volatile("fence.proxy.async.global;" ::: "memory");
-                break;
-            }
+        bool ok = true;
+        if (!primed) ok = stage(g);
+        for (int k = 0; k < nsteps; ++k) {
             const int b = g & 1;
             float2 *sS = sS0 + b * R * G::HST;
             float *sF = sF0 + b * G::FR_ * G::FST;
             float2 *sD = sD0 + b * R * G::HST;
-            // step k's rows: every thread waits for the bulk copies (bounded; a wait that gives up
-            // is reported at the barrier below, which every thread reaches)
-            bool ok = hr_tma::mbar_wait(&bar[b], (g >> 1) & 1u);
-            // ---- x pass of G_f on the s rows -> RX (the warp's own columns; the edge warps first
-            // fill the halo columns of the rows with the edge values)
-            if (IN_S) {
-                fill_halo(sS);
-                if (xlane) run_x_halo<RAD>(sS + xi * G::HST, xc0, sRX + xi * G::XST + xc0, tf);
-                __syncwarp();
-            }
             // ---- y pass of G_f: u for rows yu = R k + i - r; the moving image at x - u (every row's
             // four gathers first); the force of Eq. 1
             const float yk = (float)(R * k - RAD);
@@ -416,13 +385,19 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
             };
             if (interior_step(k)) force_rows(std::true_type());
             else force_rows(std::false_type());
-            // du rows complete; step k's s and test rows consumed by every warp
-            if (!__syncthreads_and(ok)) {   // a copy did not arrive: report, let this CTA's copies land, stop
-                if (t == 0) {
+            // this warp's du rows are written and step k's s and test rows consumed; the next step's x
+            // pass of G_f (of the next pair's first step after the last) runs before the wait for the
+            // other warps
+            __syncwarp();
+            if (lane == 0) hr_tma::mbar_arrive(&dbar);
+            const bool more = k + 1 < nsteps || (!LOOP && next_pair >= 0);
+            if (more) ok = stage(g + 1) && ok;
+            ok = hr_tma::mbar_wait(&dbar, g & 1u) && ok;
+            if (!__all_sync(0xffffffffu, ok)) {   // a wait gave up (then the other warps' do): report, let this
+                if (t == 0) {                     // CTA's copies land, stop
                     atomicExch(a.err, 1);
                     hr_tma::mbar_wait(&bar[b], (g >> 1) & 1u);
-                    if (k + 1 < nsteps || (!LOOP && next_pair >= 0))
-                        hr_tma::mbar_wait(&bar[b ^ 1], ((g + 1) >> 1) & 1u);
+                    if (more) hr_tma::mbar_wait(&bar[b ^ 1], ((g + 1) >> 1) & 1u);
                 }
                 return;
             }
@@ -441,8 +416,44 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_strip_kernel(IterArgs a, 
                 if (yu >= 0 && yu < h) run_x_halo<RAD>(sD + xi * G::HST, xc0, sDX + xi * G::XST + xc0, tu);
             }
             __syncwarp();
+            // ---- y pass of G_u over the DX window, s = u + G_u * du (DX rows of the warp's own columns).
+            // Interior steps (every row inside, none at an edge) run without the edge handling.
+            {
+                float2 *dk = dst + (ptrdiff_t)(R * k - 2 * RAD) * NT + t;   // row yo for i = 0
+                auto outputs = [&](auto interior) {
+                    constexpr bool IN = decltype(interior)::value;
+#pragma unroll
+                    for (int i = 0; i < R; ++i) {
+                        const int yu = R * k + i - RAD, yo = yu - RAD;   // du row entering, output row
+                        if (IN || yu >= 0) {
+                            const float2 v = (IN || yu < h) ? sDX[i * G::XST + t] : last_dx;
+                            if (!IN && yu < h) last_dx = v;
+                            dxw[(i + R - RAD) % R] = v;   // row yu in slot yu mod R
+                            if (!IN && yu == 0) {
+#pragma unroll
+                                for (int j = 0; j < R; ++j) dxw[j] = v;
+                            }
+                        }
+                        if (IN || (yo >= 0 && yo < h)) {
+                            // rows yo - r + j = yu - 2r + j sit in slots (i - 3r + j) mod R
+                            float2 acc = __fmul2_rn(tu[0], dxw[(i + 2 * R - 3 * RAD) % R]);
+#pragma unroll
+                            for (int j = 1; j < R; ++j) acc = ffma2(tu[j], dxw[(i + 2 * R - 3 * RAD + j) % R], acc);
+                            const float2 uo = i >= RAD ? ucur[i - RAD] : uprev[i];
+                            dk[i * NT] = __fadd2_rn(uo, acc);   // row yo
+                        }
+                    }
+                };
+                if (interior_step(k)) outputs(std::true_type());
+                else outputs(std::false_type());
+#pragma unroll
+                for (int i = 0; i < RAD; ++i) uprev[i] = ucur[R - RAD + i];
+            }
             ++g;
         }
+        primed = !LOOP && next_pair >= 0;
+        // LOOP: the next iteration's bulk copies read the rows of s_{k+1} just written (async proxy)
+        if (LOOP) asm volatile("fence.proxy.async.global;" ::: "memory");
         // SSD of the pair (one partial: the level runs with tiles = 1)
         for (int o = 16; o > 0; o >>= 1) ssd += __shfl_xor_sync(0xffffffffu, ssd, o);
         if (lane == 0) red[warp] = ssd;
