@@ -103,20 +103,8 @@ __device__ __forceinline__ void warp_cell(int q, float u, int m, int &i, float &
     i = (int)xc;
 }
 
-// warp_cell with the pixel index q and the largest cell index m - 2 given as
-// floats (integer-valued, exact): the same cell and weight.
-__device__ __forceinline__ void warp_cell_f(float q, float u, float m2, int &i, float &f)
-{
-    const float n = floorf(-u);
-    const float fr = -u - n;
-    const float x = q + n;
-    const float xc = fminf(fmaxf(x, 0.0f), m2);
-    f = __saturatef(fr + (x - xc));
-    i = (int)xc;
-}
-
-// Both axes of warp_cell_f in packed FP32x2 steps: the pixel q - u, cells c (integer-valued floats) and
-// weights f, m2 the largest cells.  With n' = ceil(u) = -floor(-u), a - b as fma(b, -1, a): the same
+// Both axes of warp_cell in packed FP32x2 steps: the point q - u, cells c and pixels q as integer-valued
+// floats, weights f, m2 the largest cells.  With n' = ceil(u) = -floor(-u), a - b as fma(b, -1, a): the same
 // rounding steps, so the same cell and weight.
 __device__ __forceinline__ void warp_cell2(float2 q, float2 u, float2 m2, float2 &c, float2 &f)
 {
@@ -841,6 +829,7 @@ __global__ void __launch_bounds__(NT_, MINB) demons_iter_tma_kernel(const __grid
 
 #include "demons_strip.cuh"
 #include "demons_level.cuh"
+#include "demons_cluster.cuh"
 
 struct CtrlArgs {
     const float *part;       // [B][tiles]
@@ -1257,6 +1246,129 @@ int launch_level(hrebsd_ctx *ctx, const lvl::LevelArgs &a, cudaStream_t st)
     return HREBSD_OK;
 }
 
+// True when the caller pinned the shape of this level size (hrebsd_set_tile_variant).
+bool hr_pinned_variant(const hrebsd_ctx *ctx, int h, int w)
+{
+    for (const auto &t : ctx->tune)
+        if (t.h == h && t.w == w) return t.pinned != 0;
+    return false;
+}
+
+constexpr int kVarNT[kTileVariants] = {256, 256, 256, 512, 768, 0, 0, 512};   // threads of a tile shape
+
+// The shape that a level's iterations run in, without the cluster form.
+struct LevelShape {
+    int var;
+    bool level, strip, tma;
+};
+
+// The cluster form of a level: CTAs per pair, rows per band, clusters resident at once.
+struct ClusterPlan {
+    int C = 0, hb = 0, st = 0, active = 0;
+    size_t smem = 0;
+    float cycles = 0.0f;   // estimated SM cycles of one iteration of the batch
+};
+constexpr size_t kClusterSmem = 222 * 1024;   // of 227 KB, the rest static
+
+int cluster_active(hrebsd_ctx *ctx, int C, int *out)
+{
+    static int configured_dev = -1;
+    static int active[clu::MAXC + 1] = {};
+    if (configured_dev != ctx->device) {
+        auto k = clu::demons_cluster_kernel;
+        HR_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmem));
+        HR_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        for (int c = 1; c <= clu::MAXC; c *= 2) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)c);
+            cfg.blockDim = dim3(clu::NT);
+            cfg.dynamicSmemBytes = kClusterSmem;
+            cudaLaunchAttribute at;
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = (unsigned)c;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                n = 0;
+            }
+            active[c] = n;
+        }
+        configured_dev = ctx->device;
+    }
+    *out = active[C];
+    return HREBSD_OK;
+}
+
+// Estimated SM cycles of one iteration of B pairs of h x w, fitted to measured levels of 20 iterations of 1
+// to 600 pairs, 23 x 25 to 256 x 256 pixels (within ~15 %).  The row sweep: 512 / w CTAs per SM, one pair
+// each, a step of 7 rows takes longer the fuller the SM is.  The tiles: the launch of the iteration and of
+// the control kernel, then the tiles' pixels.  The level in one CTA: at most two per SM.
+float shape_cycles(const hrebsd_ctx *ctx, const LevelShape &s, int B, int h, int w)
+{
+    const float sms = (float)ctx->num_sms;
+    if (s.level) {
+        const int share = (B + ctx->num_sms - 1) / ctx->num_sms;
+        return (float)((share + 1) / 2) * (2000.0f + 2.45f * (float)(h * w) * (share > 1 ? 2.0f : 1.0f));
+    }
+    if (s.strip) {
+        const float load = (float)B * (float)w / (512.0f * sms);
+        return (float)((h + 12) / 7) * (3500.0f + 2700.0f * fminf(load, 1.0f)) * fmaxf(load, 1.0f) + (load > 1.0f ? 6000.0f : 0.0f);
+    }
+    const int tx = s.tma ? kVarTX[s.var] : TX, ty = s.tma ? kVarTY[s.var] : TY;
+    const float px = (float)((w + tx - 1) / tx * tx) * (float)((h + ty - 1) / ty * ty);   // whole tiles
+    return (s.tma ? 14000.0f : 18000.0f) + (s.tma ? 3.5f : 4.0f) * (float)B * px / sms;
+}
+
+// The same for the cluster form: once for every round of resident clusters, the barriers and latencies of
+// an iteration, the band's pixels, and the regrouped SSD (group, tasks).  The best cluster size; C = 0 when
+// the level does not fit.
+int plan_cluster(hrebsd_ctx *ctx, int B, int h, int w, int group, int tasks, ClusterPlan *best)
+{
+    best->C = 0;
+    for (int C = 1; C <= clu::MAXC; C *= 2) {
+        ClusterPlan p;
+        p.C = C;
+        p.hb = (h + C - 1) / C;
+        p.st = clu::row_stride(w);
+        if ((C > 1 && p.hb < 4) || (C - 1) * p.hb >= h || (long long)(p.hb + 6) * w >= 65536) continue;
+        p.smem = clu::bytes(p.hb, w, group != clu::G_FREE);
+        if (p.smem > kClusterSmem) continue;
+        const int e = cluster_active(ctx, C, &p.active);
+        if (e) return e;
+        if (p.active < 1) continue;
+        p.cycles = C > 1 ? 6000.0f + 2.3f * (float)(p.hb * w) : 3200.0f + 1.85f * (float)(p.hb * w);
+        if (group == clu::G_STRIP) p.cycles += 2000.0f + 55.0f * (float)h;
+        else if (group != clu::G_FREE) p.cycles += 2000.0f + 2200.0f * (float)((tasks + 16 * C - 1) / (16 * C));
+        p.cycles *= (float)((B + p.active - 1) / p.active);
+        if (!best->C || p.cycles < best->cycles) *best = p;
+    }
+    return HREBSD_OK;
+}
+
+int launch_cluster(hrebsd_ctx *ctx, const clu::ClusterArgs &a, const ClusterPlan &p, cudaStream_t st)
+{
+    const int n = a.B < p.active ? a.B : p.active;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(n * p.C));
+    cfg.blockDim = dim3(clu::NT);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)p.C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = p.C > 1 ? 1 : 0;
+    hr_prof_begin(ctx, st);
+    HR_CHECK(cudaLaunchKernelEx(&cfg, clu::demons_cluster_kernel, a));
+    hr_prof_end(ctx, PROF_ITER, st);
+    HR_LAUNCHED(ctx);
+    return HREBSD_OK;
+}
+
 // Pairs the loop form keeps resident at once (one CTA each) at a level w pixels wide.
 template <int NT>
 int strip_capacity_t(hrebsd_ctx *ctx)
@@ -1648,11 +1760,66 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
         const bool use_tma = !use_level && !use_strip && rad > 0 && !ctx->no_tma && cap > 1 &&
                              encode_maps(rad, var, (const float2 *)s0, (const float2 *)s1, (const float2 *)u0, tl[l],
                                          B, h, w, tmS, &tmF);
+        // the whole level in the shared memory of a cluster per pair, where that is estimated to be faster
+        // and the caller did not pin another shape
+        ClusterPlan plan;
+        clu::ClusterArgs ca;
+        if (rad == clu::RAD && cap >= 1 && !ctx->no_tma && !hr_pinned_variant(ctx, h, w)) {
+            const LevelShape shape{var, use_level, use_strip, use_tma};
+            // the rule can end the level before the cap: the SSD has to be summed as that shape sums it
+            const bool regroup = p->stop_window > 0 && cap > p->stop_window;
+            const bool tile = !use_level && !use_strip;
+            ca.group = !regroup ? clu::G_FREE : use_level ? clu::G_LEVEL : use_strip ? clu::G_STRIP : use_tma ? clu::G_TILE : clu::G_PLAIN;
+            ca.tx = !tile ? w : use_tma ? kVarTX[var] : TX;
+            ca.ty = !tile ? h : use_tma ? kVarTY[var] : TY;
+            ca.nt = use_level ? lvl::NT : use_strip ? w : use_tma ? kVarNT[var] : kIterThreads;
+            ca.tiles_x = (w + ca.tx - 1) / ca.tx;
+            ca.tiles = ca.tiles_x * ((h + ca.ty - 1) / ca.ty);
+            ca.tasks = ca.tiles * (ca.nt / 32);
+            if (!regroup || ca.tasks <= clu::MAX_TASKS) {
+                if ((e = plan_cluster(ctx, B, h, w, ca.group, ca.tasks, &plan))) return e;
+                if (plan.C && plan.cycles > 0.9f * shape_cycles(ctx, shape, B, h, w)) plan.C = 0;
+            }
+        }
         // The launches of one level: list reset, cap x (iteration, control) -- or, in the loop
         // form, iteration 0 and its control, then one launch for the rest --, finalize,
         // prolongation.  Replayed from a cached CUDA graph when possible.
         auto emit = [&](cudaStream_t st) -> int {
             int e2;
+            if (plan.C) {
+                ca.Ftest = tl[l];
+                ca.Mref = rl[l];
+                ca.ref_idx = ref_idx;
+                ca.u0 = (const float2 *)u0;
+                ca.uout = l == 0 ? field : (float *)uout;
+                ca.hist = (double *)hist;
+                ca.iters = iters;
+                ca.status = status;
+                ca.px_count = hr_prof_pixiters(ctx);
+                ca.B = B;
+                ca.h = h;
+                ca.w = w;
+                ca.hist_stride = cap_max + 1;
+                ca.cap = cap;
+                ca.window = p->stop_window;
+                ca.level = l;
+                ca.levels = L;
+                ca.planar = l == 0;
+                ca.C = plan.C;
+                ca.hb = plan.hb;
+                ca.st = plan.st;
+                auto magic = [](int n) { return (unsigned)(((1ull << 32) + n - 1) / n); };
+                ca.mw = magic(w);
+                ca.mhb = magic(plan.hb);
+                ca.mbw = magic(ca.tx + 2 * clu::RAD);
+                ca.tol = p->stop_tol;
+                ca.alpha2 = p->alpha * p->alpha;
+                ca.taps = taps;
+                if ((e2 = launch_cluster(ctx, ca, plan, st))) return e2;
+                if (l > 0)   // to the finer level's stored size
+                    return launch_prolong(ctx, (const float2 *)uout, (float2 *)u0, B, h, w, H >> (l - 1), W >> (l - 1), st);
+                return HREBSD_OK;
+            }
             if (use_level) {   // the whole level, final field included, in one launch
                 lvl::LevelArgs a;
                 a.Ftest = tl[l];
@@ -1797,7 +1964,7 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
         static_assert(sizeof(kp) / sizeof(kp[0]) <= sizeof(key.p) / sizeof(key.p[0]), "graph key");
         for (size_t i = 0; i < sizeof(kp) / sizeof(kp[0]); ++i) key.p[i] = kp[i];
         const int ki[] = {l, L, B, h, w, cap, cap_max, rad, var, (int)use_tma, p->stop_window, (int)use_strip,
-                          (int)use_loop, (int)use_level};
+                          (int)use_loop, (int)use_level, plan.C};
         for (size_t i = 0; i < sizeof(ki) / sizeof(ki[0]); ++i) key.i[i] = ki[i];
         key.f[0] = p->alpha;
         key.f[1] = p->stop_tol;
@@ -1865,10 +2032,10 @@ extern "C" int hrebsd_set_tile_variant(hrebsd_ctx *ctx, int h, int w, int varian
     for (size_t i = 0; i < ctx->tune.size(); ++i)
         if (ctx->tune[i].h == h && ctx->tune[i].w == w) {
             if (variant < 0) ctx->tune.erase(ctx->tune.begin() + i);
-            else ctx->tune[i].var = variant;
+            else ctx->tune[i] = hr_tune_entry{h, w, variant, 1};
             return HREBSD_OK;
         }
-    if (variant >= 0) ctx->tune.push_back(hr_tune_entry{h, w, variant});
+    if (variant >= 0) ctx->tune.push_back(hr_tune_entry{h, w, variant, 1});
     return HREBSD_OK;
 }
 
@@ -2084,6 +2251,8 @@ extern "C" int hrebsd_autotune(hrebsd_ctx *ctx, int B, int H, int W, const hrebs
                 }
             }
             int e3 = hrebsd_set_tile_variant(ctx, h, w, best_v);
+            for (auto &te : ctx->tune)
+                if (te.h == h && te.w == w) te.pinned = 0;   // a measured choice, not the caller's
             if (e3) return e3;
         }
         return HREBSD_OK;

@@ -52,9 +52,9 @@ struct hr_graph_entry {
     long long nodes;          // kernel launches in the graph
     unsigned long long last;  // LRU clock
 };
-// Tile shape chosen for a level size (autotuner or caller).
+// Tile shape chosen for a level size (autotuner, or pinned by the caller).
 struct hr_tune_entry {
-    int h, w, var;
+    int h, w, var, pinned;
 };
 // Copy of a level's reference images in a CUDA array (rows R x h stacked, one array per level width)
 // behind a texture object, for the four-texel gathers of the row sweep (demons.cu).
