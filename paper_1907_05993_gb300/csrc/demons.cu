@@ -844,15 +844,32 @@ struct CtrlArgs {
     float tol;
 };
 
-// Stop rule of one level after iteration k (E_k complete in part[]).
-__global__ void demons_control_kernel(CtrlArgs c)
+// Stop rule of one level after iteration k (E_k complete in part[]): `lanes` consecutive lanes (a power of
+// two up to 32) per active pair add its tiles' partials in FP64.  One thread per pair took 14 us a launch
+// where a pair has 640 tiles (16 pairs of 1244 x 1024), 6 us with a warp.
+__global__ void __launch_bounds__(256) demons_control_kernel(CtrlArgs c, int lanes)
 {
     const int n = *c.n_active;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int p = c.active[i];
+    const int sub = threadIdx.x & (lanes - 1), step = (int)(gridDim.x * blockDim.x) / lanes;
+    // (the loop is uniform in a warp: its groups take the pairs i0 .. i0 + 32 / lanes - 1)
+    for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / lanes; i - (int)(threadIdx.x & 31) / lanes < n; i += step) {
+        const bool in = i < n;
+        const int p = in ? c.active[i] : 0;
         double E = 0.0;
-        const float *pp = c.part + (size_t)p * c.tiles;
-        for (int t = 0; t < c.tiles; ++t) E += (double)pp[t];
+        if (in) {
+            const float *pp = c.part + (size_t)p * c.tiles;
+            int t = sub;
+            for (; t + 3 * lanes < c.tiles; t += 4 * lanes) {
+                const float a0 = pp[t], a1 = pp[t + lanes], a2 = pp[t + 2 * lanes], a3 = pp[t + 3 * lanes];
+                E += (double)a0;
+                E += (double)a1;
+                E += (double)a2;
+                E += (double)a3;
+            }
+            for (; t < c.tiles; t += lanes) E += (double)pp[t];
+        }
+        for (int o = lanes / 2; o > 0; o >>= 1) E += __shfl_xor_sync(0xffffffffu, E, o);
+        if (!in || sub != 0) continue;
         double *hh = c.hist + (size_t)p * c.hist_stride;
         hh[c.k] = E;
         int32_t *it = c.iters + (size_t)p * c.levels + c.level;
@@ -1900,10 +1917,12 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
                 c.level = l;
                 c.levels = L;
                 c.tol = p->stop_tol;
-                int cgrid = (B + 255) / 256;
-                if (cgrid > ctx->num_sms * 4) cgrid = ctx->num_sms * 4;
+                int lanes = 1;   // about four partials per lane
+                while (lanes < 32 && lanes * 4 < tiles) lanes *= 2;
+                const long long groups = ((long long)B * lanes + 255) / 256;
+                const int cgrid = (int)(groups < ctx->num_sms * 4LL ? groups : ctx->num_sms * 4LL);
                 hr_prof_begin(ctx, st);
-                demons_control_kernel<<<cgrid, 256, 0, st>>>(c);
+                demons_control_kernel<<<cgrid, 256, 0, st>>>(c, lanes);
                 hr_prof_end(ctx, PROF_CTRL, st);
                 HR_LAUNCHED(ctx);
             }
