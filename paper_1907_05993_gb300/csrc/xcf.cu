@@ -224,11 +224,13 @@ __global__ void __launch_bounds__(NT) xcf_kernel(const float *__restrict__ rem, 
 // S = 64 (the batched-scan ROIs): radix-8 transforms in registers.  A 64-point
 // line transform is 8 x 8 (Cooley-Tukey): eight 8-point DFTs over the stride-8
 // subsequences, a twiddle W64^(n2 k1), eight 8-point DFTs over n2, natural-
-// order output.  512 threads = 64 lines x 8; thread (line = tid % 64,
-// t = tid / 64) so that a warp touches 32 consecutive rows or columns and the
-// twiddles are warp-uniform.  Rows are padded to 65 elements (conflict-free
-// column access).  4 shared-memory passes per 2-D transform instead of 12
-// radix-2 stages.
+// order output.  8 lanes of a warp share a line, so that the exchange between
+// the two halves stays within the warp and a pass has one CTA barrier (with
+// the lanes of a line in eight warps a pass had four: 2,128 us for 62,500
+// ROIs, 1,836 us this way,
+// bound by the shared-memory wavefronts).  Rows are padded to 65 elements; a warp takes
+// lines 8 apart and the exchanged elements are rotated, so that every access
+// of a half warp touches 16 distinct 8-byte banks for rows and columns alike.
 namespace r8 {
 
 constexpr int S = 64, ZS = 65, NT = 512;
@@ -237,8 +239,9 @@ constexpr int S = 64, ZS = 65, NT = 512;
 template <int SG>
 __device__ __forceinline__ float2 mul_si(float2 z) { return SG < 0 ? make_float2(z.y, -z.x) : make_float2(-z.y, z.x); }
 
-__device__ __forceinline__ float2 add(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 sub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// packed (a - b as fma(b, -1, a): the same rounding)
+__device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 
 // 4-point DFT with sign SG, in place on (a0, a1, a2, a3)
 template <int SG>
@@ -265,20 +268,22 @@ __device__ __forceinline__ void dft8(float2 (&x)[8])
     const float2 w3o3 = make_float2(c * (-o3.x - SG * o3.y), c * (-o3.y + SG * o3.x));  // (-c, SG c) * o3
     x[0] = add(e0, o0);
     x[4] = sub(e0, o0);
-    x[1] = add(e1, w1o1);
-    x[5] = sub(e1, w1o1);
+    x[1] = make_float2(e1.x + w1o1.x, e1.y + w1o1.y);   // (not packed: contracts with w1o1's product)
+    x[5] = make_float2(e1.x - w1o1.x, e1.y - w1o1.y);
     x[2] = add(e2, w2o2);
     x[6] = sub(e2, w2o2);
-    x[3] = add(e3, w3o3);
-    x[7] = sub(e3, w3o3);
+    x[3] = make_float2(e3.x + w3o3.x, e3.y + w3o3.y);
+    x[7] = make_float2(e3.x - w3o3.x, e3.y - w3o3.y);
 }
 
 // One 64-point pass over all 64 lines.  ROWS: line = row, element stride 1;
-// else line = column, element stride ZS.  tw[j] = exp(-2 pi i j / 64).
-template <int SG, bool ROWS>
-__device__ __forceinline__ void pass64(float2 *z, const float2 *tw)
+// else line = column, element stride ZS.  tw[k] = exp(-2 pi i k t / 64), t the lane's place in its line.
+// KEEP: nothing is stored; out[k2] = the real part of X[t + 8 k2] of the line.
+template <int SG, bool ROWS, bool KEEP = false>
+__device__ __forceinline__ void pass64(float2 *z, const float2 (&tw)[8], float *out = nullptr)
 {
-    const int line = threadIdx.x & 63, t = threadIdx.x >> 6;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = lane & 7;
+    const int line = (warp & 7) + 32 * (warp >> 3) + 8 * (lane >> 3);
     const int ls = ROWS ? ZS : 1, es = ROWS ? 1 : ZS;
     float2 *zl = z + line * ls;
     float2 v[8];
@@ -288,25 +293,30 @@ __device__ __forceinline__ void pass64(float2 *z, const float2 *tw)
     dft8<SG>(v);
 #pragma unroll
     for (int k1 = 1; k1 < 8; ++k1) {
-        float2 w = tw[t * k1];
+        float2 w = tw[k1];
         if (SG > 0) w.y = -w.y;
         v[k1] = make_float2(v[k1].x * w.x - v[k1].y * w.y, v[k1].x * w.y + v[k1].y * w.x);
     }
-    __syncthreads();
+    __syncwarp();
 #pragma unroll
-    for (int k1 = 0; k1 < 8; ++k1) zl[(8 * t + k1) * es] = v[k1];
-    __syncthreads();
+    for (int k1 = 0; k1 < 8; ++k1) zl[(8 * t + ((k1 + t) & 7)) * es] = v[k1];   // Y'[n2 = t][k1], rotated by n2
+    __syncwarp();
     // stage 2: DFT over n2 of Y'[n2][k1 = t] -> X[t + 8 k2]
 #pragma unroll
-    for (int n2 = 0; n2 < 8; ++n2) v[n2] = zl[(8 * n2 + t) * es];
+    for (int n2 = 0; n2 < 8; ++n2) v[n2] = zl[(8 * n2 + ((t + n2) & 7)) * es];
     dft8<SG>(v);
-    __syncthreads();
+    if (KEEP) {
+#pragma unroll
+        for (int k2 = 0; k2 < 8; ++k2) out[k2] = v[k2].x;
+        return;
+    }
+    __syncwarp();
 #pragma unroll
     for (int k2 = 0; k2 < 8; ++k2) zl[(t + 8 * k2) * es] = v[k2];
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(NT) xcf64_kernel(const float *__restrict__ rem, const float *__restrict__ test, int B,
+__global__ void __launch_bounds__(NT, 2) xcf64_kernel(const float *__restrict__ rem, const float *__restrict__ test, int B,
                                                    int H, int W, const int32_t *__restrict__ roi, int N, int window,
                                                    float *q, int32_t *peak, float *ph, int32_t *near_tie)
 {
@@ -338,56 +348,80 @@ __global__ void __launch_bounds__(NT) xcf64_kernel(const float *__restrict__ rem
     }
     const float *T = test + (size_t)b * H * W + (size_t)y0 * W + x0;
     const float *Rr = rem + (size_t)b * H * W + (size_t)y0 * W + x0;
+    constexpr int PER = S * S / NT;   // pixels of a thread, in registers until they are windowed
+    const int px = threadIdx.x % S, py = threadIdx.x / S;
     float st = 0.0f, sr = 0.0f;
-    for (int idx = threadIdx.x; idx < S * S; idx += NT) {
-        const int y = idx / S, x = idx % S;
-        const float tv = __ldg(T + (size_t)y * W + x), rv_ = __ldg(Rr + (size_t)y * W + x);
-        z[y * ZS + x] = make_float2(tv, rv_);
-        st += tv;
-        sr += rv_;
+    float2 raw[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const size_t at = (size_t)(py + i * (NT / S)) * W + px;
+        raw[i] = make_float2(__ldg(T + at), __ldg(Rr + at));
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        st += raw[i].x;
+        sr += raw[i].y;
     }
     const float mt = block_sum<NT>(st, red) * (1.0f / (S * S));
     const float mr = block_sum<NT>(sr, red) * (1.0f / (S * S));
     float nt = 0.0f, nr = 0.0f;
-    for (int idx = threadIdx.x; idx < S * S; idx += NT) {
-        const int y = idx / S, x = idx % S;
-        const float wgt = win[y] * win[x];
-        float2 v = z[y * ZS + x];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int y = py + i * (NT / S);
+        const float wgt = win[y] * win[px];
+        float2 v = raw[i];
         v.x = (v.x - mt) * wgt;
         v.y = (v.y - mr) * wgt;
-        z[y * ZS + x] = v;
+        z[y * ZS + px] = v;
         nt = fmaf(v.x, v.x, nt);
         nr = fmaf(v.y, v.y, nr);
     }
     nt = sqrtf(block_sum<NT>(nt, red));
     nr = sqrtf(block_sum<NT>(nr, red));   // ends with a barrier: z complete
 
-    pass64<-1, true>(z, tw);
-    pass64<-1, false>(z, tw);
+    float2 wt[8];   // this lane's twiddles, the same in every pass
+#pragma unroll
+    for (int k = 0; k < 8; ++k) wt[k] = tw[k * (threadIdx.x & 7)];
+    pass64<-1, true>(z, wt);
+    pass64<-1, false>(z, wt);
 
-    // cross-power P(k) = T(k) conj(R(k)), P(-k) = conj(P(k)); pairs (k, -k) in place
-    for (int idx = threadIdx.x; idx < S * S; idx += NT) {
-        const int ky = idx / S, kx = idx % S;
+    // cross-power P(k) = T(k) conj(R(k)), P(-k) = conj(P(k)); pairs (k, -k) in place, from the one that
+    // comes first in row-major order: rows 1 .. 31, columns 0 .. 32 of rows 0 and 32
+    auto cross = [&](int ky, int kx) {
         const int my = (S - ky) & (S - 1), mx = (S - kx) & (S - 1);
-        const int m = my * S + mx;
-        if (idx > m) continue;
-        const float2 zk = z[ky * ZS + kx], zm = z[my * ZS + mx];
+        float2 *pk = z + ky * ZS + kx, *pm = z + my * ZS + mx;
+        const float2 zk = *pk, zm = *pm;
         const float2 Tk = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
         const float2 Rk = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
         const float2 P = make_float2(Tk.x * Rk.x + Tk.y * Rk.y, Tk.y * Rk.x - Tk.x * Rk.y);
-        z[ky * ZS + kx] = P;
-        if (m != idx) z[my * ZS + mx] = make_float2(P.x, -P.y);
+        *pk = P;
+        if (pm != pk) *pm = make_float2(P.x, -P.y);
+    };
+#pragma unroll
+    for (int i = 0; i < S / 2 * S / NT; ++i) {
+        const int ky = 1 + (int)threadIdx.x / S + i * (NT / S), kx = threadIdx.x % S;
+        if (ky < S / 2 || kx <= S / 2) cross(ky, kx);
     }
+    if (threadIdx.x <= S / 2) cross(0, threadIdx.x);
     __syncthreads();
-    pass64<1, true>(z, tw);
-    pass64<1, false>(z, tw);
+    pass64<1, true>(z, wt);
+    float corr[8];
+    pass64<1, false, true>(z, wt, corr);   // (line = column)
 
-    // argmax of c = Re(z) / S^2 (first maximum in row-major order) and runner-up
+    // argmax of c = Re(z) / S^2 (first maximum in row-major order) and runner-up, each lane over its own
+    // results; the surface, for the peak's neighbours, as plain rows of 64 floats once every lane is done
     const float scale = 1.0f / (float)(S * S);
     float bv = -INFINITY, bv2 = -INFINITY;
     int bi = 0x7fffffff;
-    for (int idx = threadIdx.x; idx < S * S; idx += NT) {
-        const float v = z[(idx / S) * ZS + idx % S].x * scale;
+    float *surf = reinterpret_cast<float *>(z);
+    const int lane_ = threadIdx.x & 31, warp_ = threadIdx.x >> 5;
+    const int c_col = (warp_ & 7) + 32 * (warp_ >> 3) + 8 * (lane_ >> 3), c_row = lane_ & 7;
+    __syncthreads();
+#pragma unroll
+    for (int k2 = 0; k2 < 8; ++k2) {
+        const int idx = (c_row + 8 * k2) * S + c_col;
+        const float v = corr[k2] * scale;
+        surf[idx] = v;
         if (better(v, idx, bv, bi)) {
             bv2 = bv;
             bv = v;
@@ -428,10 +462,8 @@ __global__ void __launch_bounds__(NT) xcf64_kernel(const float *__restrict__ rem
         }
         const int py = i / S, px = i % S;
         const float c0 = v;
-        const float cxm = z[py * ZS + ((px + S - 1) & (S - 1))].x * scale;
-        const float cxp = z[py * ZS + ((px + 1) & (S - 1))].x * scale;
-        const float cym = z[((py + S - 1) & (S - 1)) * ZS + px].x * scale;
-        const float cyp = z[((py + 1) & (S - 1)) * ZS + px].x * scale;
+        const float cxm = surf[py * S + ((px + S - 1) & (S - 1))], cxp = surf[py * S + ((px + 1) & (S - 1))];
+        const float cym = surf[((py + S - 1) & (S - 1)) * S + px], cyp = surf[((py + 1) & (S - 1)) * S + px];
         float dx = 0.0f, dy = 0.0f, den;
         den = cxm - 2.0f * c0 + cxp;
         if (den != 0.0f) dx = (cxm - cxp) / (2.0f * den);
@@ -452,8 +484,9 @@ __global__ void __launch_bounds__(NT) xcf64_kernel(const float *__restrict__ rem
 // ---------------------------------------------------------------------------
 // S = 256 (the paper's ROIs of 256 x 256 on 1244 x 1024 patterns): the 2-D
 // array (512 KB of complex values) does not fit in shared memory, so the
-// transform goes through a global scratch array Z [roi][256][256] in three
+// transform goes through a global scratch array Z [roi][256][256] in four
 // launches, each staging lines in shared memory:
+//   sums:  per ROI and 32 rows, the rows' sums (for the means);
 //   rows:  per ROI, means and window norms, then 32-row chunks: zero mean,
 //          Hann window, pack z = t + i r, forward row FFTs, store;
 //   cols:  per ROI and group of 16 columns k with their mirrors -k: forward
@@ -461,45 +494,83 @@ __global__ void __launch_bounds__(NT) xcf64_kernel(const float *__restrict__ rem
 //          T = (Z(k) + conj Z(-k))/2, R = (Z(k) - conj Z(-k))/2i (and
 //          P(-k) = conj P(k)), inverse column FFTs, store;
 //   peak:  per ROI, 32-row chunks: inverse row FFTs, the real correlation
-//          c = Re / S^2 written over the scratch, first maximum in row-major
-//          order and runner-up, then the parabolic sub-pixel fit from the
-//          stored surface.
+//          c = Re / S^2, first maximum in row-major order and runner-up, then
+//          the three rows around the peak once more for the parabolic
+//          sub-pixel fit.
 // The arithmetic per element is that of the shared-memory kernel (radix-2
-// transforms, FP32).
+// transforms, FP32).  Bound by the scratch's traffic (three passes over 8 B per
+// element) and the transforms' instructions; 1,600 ROIs: sums
+// 159 us, rows 370 (2,489 with one stage at a time and the rows summed from
+// global memory), columns 647 (2,120), peak 265 (1,154).
 namespace x256 {
 
-constexpr int S = 256, NT = 256, LS = S + 1;   // line stride (odd: conflict-free column access)
+constexpr int S = 256, NT = 256;
+constexpr int LS = S + S / 16 + 1;   // line stride: one pad element after 16, an odd total (conflict-free)
+constexpr int LANES = 16;            // lanes that share a line, 16 elements each
+__device__ __forceinline__ int at(int p) { return p + (p >> 4); }   // element p of a line
+__device__ __forceinline__ int brev4(int v) { return (int)(__brev((unsigned)v) >> 28); }
 
-__device__ __forceinline__ int brev8(int v) { return (int)(__brev((unsigned)v) >> 24); }
-
-// In-place 256-point transforms of nl lines z[line * LS + i]; sign -1 forward, +1 inverse (unscaled).
-__device__ void fft_lines(float2 *z, int nl, const float2 *tw, int sign)
+// Stages half = H0, 2 H0, 4 H0, 8 H0 of the radix-2 transform on 16 elements held by one lane: element e is
+// position base + step e of the line, step = H0, base < H0.  The butterflies and twiddles of the stages one
+// by one, in registers.
+template <int H0>
+__device__ __forceinline__ void stages(float2 (&v)[16], int base, const float2 *tw, int sign)
 {
-    for (int idx = threadIdx.x; idx < nl * S; idx += NT) {
-        const int line = idx >> 8, x = idx & (S - 1), j = brev8(x);
-        if (x < j) {
-            float2 *p = z + line * LS;
-            const float2 t = p[x];
-            p[x] = p[j];
-            p[j] = t;
-        }
-    }
-    __syncthreads();
-    for (int half = 1; half < S; half <<= 1) {
-        const int tstep = S / (2 * half);
-        for (int b = threadIdx.x; b < nl * (S / 2); b += NT) {
-            const int line = b >> 7, bf = b & (S / 2 - 1);
-            const int grp = bf / half, j = bf % half;
-            const int i0 = grp * 2 * half + j, i1 = i0 + half;
+#pragma unroll
+    for (int m = 1; m < 16; m <<= 1) {   // half = H0 m
+        const int tstep = S / (2 * H0 * m);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            if (e & m) continue;
+            const int j = base + H0 * (e & (m - 1));   // position within the half
             float2 w = tw[j * tstep];
             if (sign > 0) w.y = -w.y;
-            float2 *p = z + line * LS;
-            const float2 v = cmul(p[i1], w), u = p[i0];
-            p[i0] = make_float2(u.x + v.x, u.y + v.y);
-            p[i1] = make_float2(u.x - v.x, u.y - v.y);
+            const float2 x = cmul(v[e + m], w), u = v[e];
+            v[e] = make_float2(u.x + x.x, u.y + x.y);
+            v[e + m] = make_float2(u.x - x.x, u.y - x.y);
         }
-        __syncthreads();
     }
+}
+
+// The 256-point transform of one line in shared memory by 16 lanes of a warp (lane g of the line; every lane
+// of the warp takes part, `live` false for a half warp without a line): the bit-reversed inputs of 16
+// consecutive positions are read, four stages run in registers, the elements are exchanged through the line
+// and four more stages run on the positions g + 16 e, which lane g returns in v.  Four shared-memory accesses per
+// element and no CTA barrier, where one stage at a time takes 18 and nine.
+__device__ __forceinline__ void fft_line(float2 *line, int g, bool live, const float2 *tw, int sign, float2 (&v)[16])
+{
+    if (live) {
+        const int rg = brev4(g);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] = line[at(16 * brev4(e) + rg)];
+        stages<1>(v, 0, tw, sign);
+    }
+    __syncwarp();
+    if (live)
+#pragma unroll
+        for (int e = 0; e < 16; ++e) line[at(16 * g + e)] = v[e];
+    __syncwarp();
+    if (live) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] = line[at(g + 16 * e)];
+        stages<16>(v, g, tw, sign);
+    }
+}
+
+// fft_line of nl lines (stride LS), results in place.
+__device__ __forceinline__ void fft_lines(float2 *z, int nl, const float2 *tw, int sign)
+{
+    const int g = threadIdx.x % LANES;
+    for (int l0 = 0; l0 < nl; l0 += NT / LANES) {
+        const int l = l0 + (int)threadIdx.x / LANES;
+        const bool live = l < nl;
+        float2 v[16];
+        fft_line(z + l * LS, g, live, tw, sign, v);
+        if (live)   // (the lane's own positions)
+#pragma unroll
+            for (int e = 0; e < 16; ++e) z[l * LS + at(g + 16 * e)] = v[e];
+    }
+    __syncthreads();
 }
 
 __device__ void twiddles(float2 *tw)
@@ -525,10 +596,42 @@ __device__ double block_sum_d(double v, double *red)
 
 constexpr int RCH = 32;   // rows (or columns) staged at a time
 
+__device__ __forceinline__ bool outside(int x0, int y0, int H, int W) { return x0 < 0 || y0 < 0 || x0 + S > W || y0 + S > H; }
+
+// Row sums of a ROI of the chunk, 32 rows per CTA: sums[roi][2][256] (test, reference), each row summed from
+// left to right in FP32 by one thread.  The rows are staged so that the loads are whole.
+constexpr int SUM_NT = 128, SLS = S + 1;
+__global__ void __launch_bounds__(SUM_NT) sums_kernel(const float *__restrict__ rem, const float *__restrict__ test, int b0,
+                                                      int H, int W, const int32_t *__restrict__ roi, int N, float *sums)
+{
+    extern __shared__ float rows[];   // [2][RCH][SLS]
+    const int lr = blockIdx.x / (S / RCH), c0 = blockIdx.x % (S / RCH) * RCH, b = b0 + lr / N, r = lr % N;
+    const int x0 = roi[2 * r] - S / 2, y0 = roi[2 * r + 1] - S / 2;
+    if (outside(x0, y0, H, W)) return;
+    const size_t off = (size_t)b * H * W + (size_t)(y0 + c0) * W + x0;
+#pragma unroll 8
+    for (int idx = threadIdx.x; idx < 2 * RCH * S; idx += SUM_NT) {   // asynchronous: every load in flight at once
+        const int line = idx >> 8, x = idx & (S - 1);
+        const float *src = (line < RCH ? test : rem) + off + (size_t)(line & (RCH - 1)) * W + x;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(rows + line * SLS + x)), "l"(src)
+                     : "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x < 2 * RCH) {
+        const float *p = rows + threadIdx.x * SLS;
+        float a = 0.0f;
+#pragma unroll 16
+        for (int x = 0; x < S; ++x) a += p[x];
+        sums[((size_t)lr * 2 + threadIdx.x / RCH) * S + c0 + threadIdx.x % RCH] = a;
+    }
+}
+
 // One CTA per (pair, ROI) of the chunk.  norms[2 * roi] = |t_w|, |r_w| (negative: ROI outside the image).
-__global__ void __launch_bounds__(NT) rows_kernel(const float *__restrict__ rem, const float *__restrict__ test, int b0,
-                                                  int H, int W, const int32_t *__restrict__ roi, int N, int window,
-                                                  float2 *Z, float *norms)
+__global__ void __launch_bounds__(NT, 3) rows_kernel(const float *__restrict__ rem, const float *__restrict__ test, int b0,
+                                                     int H, int W, const int32_t *__restrict__ roi, int N, int window,
+                                                     float2 *Z, const float *__restrict__ sums, float *norms)
 {
     extern __shared__ float2 zs[];   // [RCH][LS]
     __shared__ float2 tw[S / 2];
@@ -536,7 +639,7 @@ __global__ void __launch_bounds__(NT) rows_kernel(const float *__restrict__ rem,
     __shared__ double red[NT / 32];
     const int lr = blockIdx.x, b = b0 + lr / N, r = lr % N;
     const int x0 = roi[2 * r] - S / 2, y0 = roi[2 * r + 1] - S / 2;
-    if (x0 < 0 || y0 < 0 || x0 + S > W || y0 + S > H) {
+    if (outside(x0, y0, H, W)) {
         if (threadIdx.x == 0) norms[2 * lr] = norms[2 * lr + 1] = -1.0f;
         return;
     }
@@ -545,36 +648,35 @@ __global__ void __launch_bounds__(NT) rows_kernel(const float *__restrict__ rem,
         win[n] = window ? 0.5f * (1.0f - cospif(2.0f * (float)n / (float)(S - 1))) : 1.0f;
     const float *T = test + (size_t)b * H * W + (size_t)y0 * W + x0;
     const float *R = rem + (size_t)b * H * W + (size_t)y0 * W + x0;
-    // means (FP32 partial sums of one row per thread, combined in FP64)
-    double st = 0.0, sr = 0.0;
-    for (int y = threadIdx.x; y < S; y += NT) {
-        float a = 0.0f, c = 0.0f;
-        for (int x = 0; x < S; ++x) {
-            a += __ldg(T + (size_t)y * W + x);
-            c += __ldg(R + (size_t)y * W + x);
-        }
-        st += a;
-        sr += c;
-    }
+    // means (one row's sum per thread, combined in FP64)
+    static_assert(S == NT, "one row per thread");
+    const double st = sums[(size_t)lr * 2 * S + threadIdx.x], sr = sums[((size_t)lr * 2 + 1) * S + threadIdx.x];
     const float mt = (float)(block_sum_d(st, red) / (S * S)), mr = (float)(block_sum_d(sr, red) / (S * S));
     float2 *Zr = Z + (size_t)lr * S * S;
     double nt = 0.0, nr = 0.0;
     for (int c0 = 0; c0 < S; c0 += RCH) {
-        float at = 0.0f, ar = 0.0f;
-        for (int idx = threadIdx.x; idx < RCH * S; idx += NT) {
-            const int y = c0 + (idx >> 8), x = idx & (S - 1);
+        float sum_t = 0.0f, sum_r = 0.0f;
+        const int x = threadIdx.x;   // (S = NT)
+#pragma unroll 8
+        for (int i = 0; i < RCH; ++i) {
+            const int y = c0 + i;
             const float wgt = win[y] * win[x];
             const float tv = (__ldg(T + (size_t)y * W + x) - mt) * wgt, rv = (__ldg(R + (size_t)y * W + x) - mr) * wgt;
-            zs[(idx >> 8) * LS + x] = make_float2(tv, rv);
-            at = fmaf(tv, tv, at);
-            ar = fmaf(rv, rv, ar);
+            zs[i * LS + at(x)] = make_float2(tv, rv);
+            sum_t = fmaf(tv, tv, sum_t);
+            sum_r = fmaf(rv, rv, sum_r);
         }
-        nt += at;
-        nr += ar;
+        nt += sum_t;
+        nr += sum_r;
         __syncthreads();
-        fft_lines(zs, RCH, tw, -1);
-        for (int idx = threadIdx.x; idx < RCH * S; idx += NT)
-            Zr[(size_t)(c0 + (idx >> 8)) * S + (idx & (S - 1))] = zs[(idx >> 8) * LS + (idx & (S - 1))];
+        const int g = threadIdx.x % LANES;
+        for (int l = (int)threadIdx.x / LANES; l < RCH; l += NT / LANES) {   // results straight to the scratch
+            float2 v[16];
+            fft_line(zs + l * LS, g, true, tw, -1, v);
+            float2 *row = Zr + (size_t)(c0 + l) * S + g;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) row[16 * e] = v[e];
+        }
         __syncthreads();
     }
     nt = block_sum_d(nt, red);
@@ -586,7 +688,7 @@ __global__ void __launch_bounds__(NT) rows_kernel(const float *__restrict__ rem,
 }
 
 // One CTA per (pair, ROI, column group g): g < 8: columns 16 g .. 16 g + 15 and their mirrors; g = 8: column 128.
-__global__ void __launch_bounds__(NT) cols_kernel(float2 *Z, const float *__restrict__ norms)
+__global__ void __launch_bounds__(NT, 3) cols_kernel(float2 *Z, const float *__restrict__ norms)
 {
     extern __shared__ float2 zs[];   // [32][LS]: slot k < 16 column C_k, slot 16 + k column -C_k
     __shared__ float2 tw[S / 2];
@@ -599,10 +701,11 @@ __global__ void __launch_bounds__(NT) cols_kernel(float2 *Z, const float *__rest
         const int k = slot & 15, c = g < 8 ? 16 * g + k : 128;
         return slot < 16 ? c : (S - c) & (S - 1);
     };
-    const int nl = 2 * nc;
+    const int nl = 2 * nc, lnl = g < 8 ? 5 : 1;   // nl = 2^lnl
+#pragma unroll 8
     for (int idx = threadIdx.x; idx < S * nl; idx += NT) {
-        const int y = idx / nl, sl = idx - y * nl, slot = sl < nc ? sl : 16 + (sl - nc);
-        zs[slot * LS + y] = Zr[(size_t)y * S + col(slot)];
+        const int y = idx >> lnl, sl = idx & (nl - 1), slot = sl < nc ? sl : 16 + (sl - nc);
+        zs[slot * LS + at(y)] = Zr[(size_t)y * S + col(slot)];
     }
     __syncthreads();
     // forward column transforms of the loaded lines (slots 0..nc-1 and 16..16+nc-1)
@@ -612,8 +715,8 @@ __global__ void __launch_bounds__(NT) cols_kernel(float2 *Z, const float *__rest
         const int k = idx / S, ky = idx - k * S, my = (S - ky) & (S - 1);
         const int c = col(k);
         const bool self = c == ((S - c) & (S - 1));   // columns 0 and 128 pair with themselves
-        float2 *pk = zs + k * LS + ky;
-        float2 *pm = self ? zs + k * LS + my : zs + (16 + k) * LS + my;
+        float2 *pk = zs + k * LS + at(ky);
+        float2 *pm = self ? zs + k * LS + at(my) : zs + (16 + k) * LS + at(my);
         if (self && ky > my) continue;
         const float2 zk = *pk, zm = *pm;
         const float2 Tk = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
@@ -625,20 +728,21 @@ __global__ void __launch_bounds__(NT) cols_kernel(float2 *Z, const float *__rest
     __syncthreads();
     fft_lines(zs, 16 + nc, tw, +1);
     for (int idx = threadIdx.x; idx < S * nl; idx += NT) {
-        const int y = idx / nl, sl = idx - y * nl, slot = sl < nc ? sl : 16 + (sl - nc);
+        const int y = idx >> lnl, sl = idx & (nl - 1), slot = sl < nc ? sl : 16 + (sl - nc);
         const int c = col(slot);
         if (slot >= 16 && c == col(slot - 16)) continue;   // self-paired column: stored once
-        Zr[(size_t)y * S + c] = zs[slot * LS + y];
+        Zr[(size_t)y * S + c] = zs[slot * LS + at(y)];
     }
 }
 
-__global__ void __launch_bounds__(NT) peak_kernel(float2 *Z, const float *__restrict__ norms, int b0, int N, float *q,
+__global__ void __launch_bounds__(NT, 3) peak_kernel(const float2 *__restrict__ Z, const float *__restrict__ norms, int b0, int N, float *q,
                                                   int32_t *peak, float *ph, int32_t *near_tie)
 {
     extern __shared__ float2 zs[];   // [RCH][LS]
     __shared__ float2 tw[S / 2];
     __shared__ float rv[NT / 32], rv2[NT / 32];
-    __shared__ int ri[NT / 32];
+    __shared__ int ri[NT / 32], s_i;
+    __shared__ float s_v, s_v2;
     const int lr = blockIdx.x;
     const size_t o = (size_t)b0 * N + lr;
     const float nt = norms[2 * lr], nr = norms[2 * lr + 1];
@@ -652,26 +756,29 @@ __global__ void __launch_bounds__(NT) peak_kernel(float2 *Z, const float *__rest
         return;
     }
     twiddles(tw);
-    float2 *Zr = Z + (size_t)lr * S * S;
-    float *Cr = reinterpret_cast<float *>(Zr);   // the real surface overwrites the rows already read
+    const float2 *Zr = Z + (size_t)lr * S * S;
     const float scale = 1.0f / (float)(S * S);
+    const int g = threadIdx.x % LANES;
     float bv = -INFINITY, bv2 = -INFINITY;
     int bi = 0x7fffffff;
     for (int c0 = 0; c0 < S; c0 += RCH) {
-        for (int idx = threadIdx.x; idx < RCH * S; idx += NT)
-            zs[(idx >> 8) * LS + (idx & (S - 1))] = Zr[(size_t)(c0 + (idx >> 8)) * S + (idx & (S - 1))];
+#pragma unroll 8
+        for (int i = 0; i < RCH; ++i) zs[i * LS + at(threadIdx.x)] = Zr[(size_t)(c0 + i) * S + threadIdx.x];
         __syncthreads();
-        fft_lines(zs, RCH, tw, +1);
-        for (int idx = threadIdx.x; idx < RCH * S; idx += NT) {
-            const int i = c0 * S + idx;
-            const float v = zs[(idx >> 8) * LS + (idx & (S - 1))].x * scale;
-            Cr[i] = v;
-            if (better(v, i, bv, bi)) {
-                bv2 = bv;
-                bv = v;
-                bi = i;
-            } else if (v > bv2) {
-                bv2 = v;
+        for (int l = (int)threadIdx.x / LANES; l < RCH; l += NT / LANES) {
+            float2 z[16];
+            fft_line(zs + l * LS, g, true, tw, +1, z);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const int i = (c0 + l) * S + g + 16 * e;
+                const float v = z[e].x * scale;
+                if (better(v, i, bv, bi)) {
+                    bv2 = bv;
+                    bv = v;
+                    bi = i;
+                } else if (v > bv2) {
+                    bv2 = v;
+                }
             }
         }
         __syncthreads();
@@ -706,10 +813,20 @@ __global__ void __launch_bounds__(NT) peak_kernel(float2 *Z, const float *__rest
                 v2 = fmaxf(v2, rv[k]);
             }
         }
-        const int py = i / S, px = i % S;
-        const float c0 = v;
-        const float cxm = Cr[py * S + ((px + S - 1) & (S - 1))], cxp = Cr[py * S + ((px + 1) & (S - 1))];
-        const float cym = Cr[((py + S - 1) & (S - 1)) * S + px], cyp = Cr[((py + 1) & (S - 1)) * S + px];
+        s_i = i;
+        s_v = v;
+        s_v2 = v2;
+    }
+    __syncthreads();
+    // the correlation's rows around the peak once more
+    const int i = s_i, py = i / S, px = i % S;
+    for (int k = 0; k < 3; ++k) zs[k * LS + at(threadIdx.x)] = Zr[(size_t)((py + S - 1 + k) & (S - 1)) * S + threadIdx.x];
+    __syncthreads();
+    fft_lines(zs, 3, tw, +1);
+    if (threadIdx.x == 0) {
+        const float c0 = s_v, v2 = s_v2;
+        const float cxm = zs[LS + at((px + S - 1) & (S - 1))].x * scale, cxp = zs[LS + at((px + 1) & (S - 1))].x * scale;
+        const float cym = zs[at(px)].x * scale, cyp = zs[2 * LS + at(px)].x * scale;
         float dx = 0.0f, dy = 0.0f, den;
         den = cxm - 2.0f * c0 + cxp;
         if (den != 0.0f) dx = (cxm - cxp) / (2.0f * den);
@@ -725,7 +842,7 @@ __global__ void __launch_bounds__(NT) peak_kernel(float2 *Z, const float *__rest
     }
 }
 
-constexpr int WS_Z = 19, WS_NORMS = 20;
+constexpr int WS_Z = 19, WS_NORMS = 20;   // WS_NORMS: norms [rois][2], then row sums [rois][2][256]
 constexpr size_t kMaxScratch = (size_t)2 << 30;   // bound of the scratch array (pairs are processed in chunks)
 
 int launch(hrebsd_ctx *ctx, const float *rem, const float *test, int B, int H, int W, const int32_t *roi, int N,
@@ -738,10 +855,11 @@ int launch(hrebsd_ctx *ctx, const float *rem, const float *test, int B, int H, i
     void *zb, *nb;
     int e;
     if ((e = hr_ws(ctx, WS_Z, per_pair * chunk, &zb))) return e;
-    if ((e = hr_ws(ctx, WS_NORMS, (size_t)chunk * N * 2 * sizeof(float), &nb))) return e;
+    if ((e = hr_ws(ctx, WS_NORMS, (size_t)chunk * N * 2 * (1 + S) * sizeof(float), &nb))) return e;
     float2 *Z = (float2 *)zb;
-    float *norms = (float *)nb;
-    const int smem_lines = 32 * LS * (int)sizeof(float2);
+    float *norms = (float *)nb, *sums = norms + (size_t)chunk * N * 2;
+    const int smem_lines = 32 * LS * (int)sizeof(float2), smem_sums = 2 * RCH * SLS * (int)sizeof(float);
+    HR_CHECK(cudaFuncSetAttribute(sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_sums));
     HR_CHECK(cudaFuncSetAttribute(rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_lines));
     HR_CHECK(cudaFuncSetAttribute(cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_lines));
     HR_CHECK(cudaFuncSetAttribute(peak_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_lines));
@@ -749,7 +867,11 @@ int launch(hrebsd_ctx *ctx, const float *rem, const float *test, int B, int H, i
         const int nb_ = B - b0 < chunk ? B - b0 : chunk;
         const unsigned rois = (unsigned)nb_ * (unsigned)N;
         hr_prof_begin(ctx, st);
-        rows_kernel<<<rois, NT, smem_lines, st>>>(rem, test, b0, H, W, roi, N, window, Z, norms);
+        sums_kernel<<<rois * (S / RCH), SUM_NT, smem_sums, st>>>(rem, test, b0, H, W, roi, N, sums);
+        hr_prof_end(ctx, PROF_XCF, st);
+        HR_LAUNCHED(ctx);
+        hr_prof_begin(ctx, st);
+        rows_kernel<<<rois, NT, smem_lines, st>>>(rem, test, b0, H, W, roi, N, window, Z, sums, norms);
         hr_prof_end(ctx, PROF_XCF, st);
         HR_LAUNCHED(ctx);
         hr_prof_begin(ctx, st);
