@@ -64,6 +64,12 @@ struct hr_mtex {
     unsigned long long tex;
 };
 
+// Inverse Gram matrix of the background quadric's basis at a pattern size (preprocess.cu).
+struct hr_quadric {
+    int H, W;
+    double ginv[36];
+};
+
 struct hrebsd_ctx {
     int device = 0;
     int num_sms = 0;
@@ -82,6 +88,7 @@ struct hrebsd_ctx {
     std::vector<hr_graph_entry> graph_cache;
     unsigned long long graph_clock = 0;
     std::vector<hr_tune_entry> tune;
+    std::vector<hr_quadric> quadrics;   // the latest pattern sizes, at most 8
     int *d_err = nullptr;   // device flag: a bounded wait gave up (static device symbol)
     hr_cnn_net *cnn = nullptr;   // learned initialiser (allocated on first use)
     double prof_ms[HREBSD_PROF_CLASSES] = {};

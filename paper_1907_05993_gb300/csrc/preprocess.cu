@@ -6,8 +6,13 @@
 // quadric once (float-float) writing the quotient less a constant to the
 // output, then reads that back for the variance and the normalised output;
 // the pattern (at most a few hundred KB) stays in L2 between the passes, so
-// HBM sees about one read and one write per pixel.
+// HBM sees between one read and one write per pixel and twice that (the CTAs'
+// patterns together exceed L2).  Bound by instruction issue (188 per pixel, a
+// third of them float-float arithmetic): 4,096 patterns of 256 x 256 1.59 ms,
+// 2.40 ms with one load in flight per thread, an integer division per pixel
+// and pass and the chunk sums in FP64.
 #include <math.h>
+#include <string.h>
 
 #include "internal.cuh"
 
@@ -17,6 +22,7 @@ constexpr int kPreThreads = 512;
 
 struct QuadricInverse {
     double ginv[36];   // inverse Gram matrix of the basis {1, x, y, x^2, xy, y^2}
+    unsigned mw;       // ceil(2^32 / W): p / W = umulhi(p, mw) while p W < 2^32
 };
 
 __device__ __forceinline__ void basis6(float x, float y, float *phi)
@@ -29,23 +35,47 @@ __device__ __forceinline__ void basis6(float x, float y, float *phi)
     phi[5] = y * y;
 }
 
-// Block-wide sum of `n` doubles per thread (n <= 6); result broadcast.
+// Block-wide sum of NV doubles per thread (NV <= 8); result broadcast.  Each exchange of the warp tree
+// halves the values a lane carries (the pairs that are added stay those of a butterfly), so that six
+// values cost 9 FP64 additions instead of 30.
 template <int NV>
 __device__ void block_sum(double (&v)[NV], double *red /* [32][NV] */)
 {
+    constexpr int P2 = NV > 4 ? 8 : NV > 2 ? 4 : NV;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    // sums over the warp; lane 32 k / P2 ends with value k
+    auto warp_sum = [&](double (&x)[P2]) {
+        int n = P2;
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-        for (int k = 0; k < NV; ++k) red[wid * NV + k] = v[k];
+        for (int o = 16; o > 0; o >>= 1) {
+            const bool up = (lane & o) != 0;
+            if (n > 1) {
+                n /= 2;
+#pragma unroll
+                for (int k = 0; k < P2 / 2; ++k)
+                    if (k < n) {
+                        const double give = up ? x[k] : x[k + n], keep = up ? x[k + n] : x[k];
+                        x[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                    }
+            } else {
+                x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+            }
+        }
+    };
+    const int mine = lane * P2 / 32;   // the value that this lane ends with
+    const bool owner = lane % (32 / P2) == 0 && mine < NV;
+    double x[P2];
+#pragma unroll
+    for (int k = 0; k < P2; ++k) x[k] = k < NV ? v[k] : 0.0;
+    warp_sum(x);
+    if (owner) red[wid * NV + mine] = x[0];
     __syncthreads();
     if (wid == 0) {
-        for (int k = 0; k < NV; ++k) {
-            double t = lane < nw ? red[lane * NV + k] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) red[k] = t;
-        }
+#pragma unroll
+        for (int k = 0; k < P2; ++k) x[k] = k < NV && lane < nw ? red[lane * NV + k] : 0.0;
+        __syncwarp();
+        warp_sum(x);
+        if (owner) red[mine] = x[0];
     }
     __syncthreads();
 #pragma unroll
@@ -92,6 +122,22 @@ __device__ __forceinline__ ff ff_mul(ff a, ff b)
     return two_sum(p, e);
 }
 
+// A running sum of FP32 terms in three parts with exact carries (~72 bits): what a sum in FP64 holds,
+// without the FP64 pipe (2 lanes per clock and SM), which bounded this kernel when every chunk's sums
+// were converted and added there.
+struct Sum3 {
+    float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+    __device__ __forceinline__ void add(float v)
+    {
+        const ff a = two_sum(s0, v);
+        s0 = a.hi;
+        const ff b = two_sum(s1, a.lo);
+        s1 = b.hi;
+        s2 = __fadd_rn(s2, b.lo);
+    }
+    __device__ __forceinline__ double value() const { return (double)s0 + ((double)s1 + (double)s2); }
+};
+
 // coordinate (2 k + 1 - n) / n in [-1, 1] of pixel k of n as hi + lo
 __device__ __forceinline__ ff pixel_coord(int k, int n)
 {
@@ -103,7 +149,7 @@ __device__ __forceinline__ ff pixel_coord(int k, int n)
 
 constexpr int kMaxDim = 1536;   // largest H and W of the background fit (per-row and per-column terms in shared memory)
 
-__global__ void __launch_bounds__(kPreThreads) preprocess_kernel(const float *__restrict__ in, float *out, int H,
+__global__ void __launch_bounds__(kPreThreads, 3) preprocess_kernel(const float *__restrict__ in, float *out, int H,
                                                                  int W, int flat, QuadricInverse qi)
 {
     __shared__ double red[32 * 6];
@@ -113,10 +159,11 @@ __global__ void __launch_bounds__(kPreThreads) preprocess_kernel(const float *__
     __shared__ float rowY[kMaxDim];                   // per row: y (the correctly rounded FP32 coordinate)
     const size_t base = (size_t)blockIdx.x * H * W;
     const float *img = in + base;
+    auto row_of = [&](int p) { return (int)__umulhi((unsigned)p, qi.mw); };
     const int n = H * W;
 
-    // Sums are taken in FP32 over chunks of kChunk pixels of one thread and the chunk sums added in
-    // FP64: the quadric's coefficients come out of a poorly conditioned 6 x 6 system, and plain FP32
+    // Sums are taken in FP32 over chunks of kChunk pixels of one thread, the chunk sums added exactly and
+    // the threads' sums in FP64: the quadric's coefficients come out of a poorly conditioned 6 x 6 system, and plain FP32
     // sums of ~128 terms would move the output by ~1e-4.
     constexpr int kChunk = 8;
     if (flat) {   // the pixel coordinates, once per row and column
@@ -127,28 +174,36 @@ __global__ void __launch_bounds__(kPreThreads) preprocess_kernel(const float *__
         for (int i = threadIdx.x; i < H; i += blockDim.x) rowY[i] = pixel_coord(i, H).hi;
         __syncthreads();
     }
+    // A chunk's pixels are loaded before any of them is used (past the end: the last pixel, counted as 0),
+    // so that a thread has kChunk loads in flight: the passes are bound by memory latency otherwise.
+    const int bd = blockDim.x;
+    auto load = [&](const float *src, int p0, float (&v)[kChunk]) {
+#pragma unroll
+        for (int c = 0; c < kChunk; ++c) v[c] = src[min(p0 + c * bd, n - 1)];
+    };
     // pass 1: quadric moments b_k = sum phi_k I (basis at the correctly rounded pixel coordinates);
     // b_0 is the pattern's sum
     double total = 0.0;
     if (flat) {
-        double d[6] = {0, 0, 0, 0, 0, 0};
+        Sum3 part[6];
         for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * blockDim.x) {
-            float acc[6] = {0, 0, 0, 0, 0, 0};
+            float acc[6] = {0, 0, 0, 0, 0, 0}, v[kChunk];
+            load(img, p0, v);
 #pragma unroll
             for (int c = 0; c < kChunk; ++c) {
-                const int p = p0 + c * blockDim.x;
-                if (p < n) {
-                    const int i = p / W, j = p - i * W;
-                    float phi[6];
-                    basis6(colX[j].x, rowY[i], phi);
-                    const float v = img[p];
+                const int p = min(p0 + c * bd, n - 1), i = row_of(p), j = p - i * W;
+                const float vc = p0 + c * bd < n ? v[c] : 0.0f;
+                float phi[6];
+                basis6(colX[j].x, rowY[i], phi);
 #pragma unroll
-                    for (int k = 0; k < 6; ++k) acc[k] = fmaf(phi[k], v, acc[k]);
-                }
+                for (int k = 0; k < 6; ++k) acc[k] = fmaf(phi[k], vc, acc[k]);
             }
 #pragma unroll
-            for (int k = 0; k < 6; ++k) d[k] += (double)acc[k];
+            for (int k = 0; k < 6; ++k) part[k].add(acc[k]);
         }
+        double d[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) d[k] = part[k].value();
         block_sum<6>(d, red);
         total = d[0];
         if (threadIdx.x == 0) {
@@ -173,7 +228,7 @@ __global__ void __launch_bounds__(kPreThreads) preprocess_kernel(const float *__
 
     // the quadric at pixel p as hi + lo: A(y) + x (B(y) + x c3)
     auto fit_at = [&](int p) -> ff {
-        const int i = p / W, j = p - i * W;
+        const int i = row_of(p), j = p - i * W;
         const ff x = {colX[j].x, colX[j].y};
         const ff A = {rowA[i].x, rowA[i].y}, Bc = {rowB[i].x, rowB[i].y};
         return ff_add(A, ff_mul(x, ff_add(Bc, ff_mul(x, C))));
@@ -183,8 +238,9 @@ __global__ void __launch_bounds__(kPreThreads) preprocess_kernel(const float *__
     bool use_fit = flat;
     if (flat) {
         bool bad = false;
+#pragma unroll 4
         for (int p = threadIdx.x; p < n; p += blockDim.x) {
-            const int i = p / W, j = p - i * W;
+            const int i = row_of(p), j = p - i * W;
             const float x = colX[j].x;
             bad |= !(fmaf(x, fmaf(x, C.hi, rowB[i].x), rowA[i].x) > 0.0f);
         }
@@ -195,8 +251,7 @@ __global__ void __launch_bounds__(kPreThreads) preprocess_kernel(const float *__
     // from the correctly rounded reciprocal), the remainder v - q f.hi exact by fma, then the
     // correction (remainder - q f.lo) / f; with the division by f.hi a product with the same
     // reciprocal (its error lands ~2^-24 below the correction, itself ~2^-24 below q)
-    auto value = [&](int p) -> ff {
-        const float v = img[p];
+    auto value = [&](int p, float v) -> ff {
         if (!use_fit) return {v, 0.0f};
         const ff f = fit_at(p);
         const float rf = __frcp_rn(f.hi);
@@ -211,58 +266,62 @@ __global__ void __launch_bounds__(kPreThreads) preprocess_kernel(const float *__
     // is stored in the output (the pattern is read before it is overwritten, by the same thread) and
     // summed for the mean
     if (!flat) {   // the raw pattern's sum for K
-        double t[1] = {0.0};
+        Sum3 part;
         for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * blockDim.x) {
-            float sv = 0.0f;
+            float sv = 0.0f, v[kChunk];
+            load(img, p0, v);
 #pragma unroll
-            for (int c = 0; c < kChunk; ++c) {
-                const int p = p0 + c * blockDim.x;
-                if (p < n) sv += img[p];
-            }
-            t[0] += (double)sv;
+            for (int c = 0; c < kChunk; ++c) sv += p0 + c * bd < n ? v[c] : 0.0f;
+            part.add(sv);
         }
+        double t[1] = {part.value()};
         block_sum<1>(t, red);
         total = t[0];
     }
     const float K = use_fit ? 1.0f : (float)(total / n);
     float *o = out + base;
-    double m[1] = {0.0};
+    Sum3 sum_d;
     for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * blockDim.x) {
-        float sd = 0.0f;
+        float sd = 0.0f, v[kChunk];
+        load(img, p0, v);
 #pragma unroll
         for (int c = 0; c < kChunk; ++c) {
-            const int p = p0 + c * blockDim.x;
-            if (p < n) {
-                const ff q = value(p);
-                const float d = __fadd_rn(__fsub_rn(q.hi, K), q.lo);
-                o[p] = d;
-                sd += d;
-            }
+            const int p = min(p0 + c * bd, n - 1);
+            const ff q = value(p, v[c]);
+            const float d = __fadd_rn(__fsub_rn(q.hi, K), q.lo);
+            if (p0 + c * bd < n) o[p] = d;
+            sd += p0 + c * bd < n ? d : 0.0f;
         }
-        m[0] += (double)sd;
+        sum_d.add(sd);
     }
+    double m[1] = {sum_d.value()};
     block_sum<1>(m, red);
     const double mean_d = m[0] / n, mean = mean_d + (double)K;
     const float md = (float)mean_d;
     // pass 3: variance about the mean
-    double v2[1] = {0.0};
+    Sum3 sum_v;
     for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * blockDim.x) {
-        float ss = 0.0f;
+        float ss = 0.0f, v[kChunk];
+        load(o, p0, v);
 #pragma unroll
         for (int c = 0; c < kChunk; ++c) {
-            const int p = p0 + c * blockDim.x;
-            if (p < n) {
-                const float d = __fsub_rn(o[p], md);
-                ss = fmaf(d, d, ss);
-            }
+            const float d = p0 + c * bd < n ? __fsub_rn(v[c], md) : 0.0f;
+            ss = fmaf(d, d, ss);
         }
-        v2[0] += (double)ss;
+        sum_v.add(ss);
     }
+    double v2[1] = {sum_v.value()};
     block_sum<1>(v2, red);
     const double sdv = sqrt(v2[0] / n);
     const float inv = (sdv > 0.0 && sdv > 1e-6 * fabs(mean)) ? (float)(1.0 / sdv) : 0.0f;
     // pass 4: output
-    for (int p = threadIdx.x; p < n; p += blockDim.x) o[p] = __fsub_rn(o[p], md) * inv;
+    for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * bd) {
+        float v[kChunk];
+        load(o, p0, v);
+#pragma unroll
+        for (int c = 0; c < kChunk; ++c)
+            if (p0 + c * bd < n) o[p0 + c * bd] = __fsub_rn(v[c], md) * inv;
+    }
 }
 
 // One pyramid level down: the 2x2 box mean, floor(H/2) x floor(W/2) (an odd
@@ -298,8 +357,10 @@ int quadric_inverse(int H, int W, QuadricInverse *qi)
             double x = (j + 0.5) / W * 2.0 - 1.0, y = (i + 0.5) / H * 2.0 - 1.0;
             double phi[6] = {1.0, x, y, x * x, x * y, y * y};
             for (int k = 0; k < 6; ++k)
-                for (int l = 0; l < 6; ++l) G[k * 6 + l] += phi[k] * phi[l];
+                for (int l = k; l < 6; ++l) G[k * 6 + l] += phi[k] * phi[l];
         }
+    for (int k = 0; k < 6; ++k)
+        for (int l = 0; l < k; ++l) G[k * 6 + l] = G[l * 6 + k];
     // Gauss-Jordan inversion with partial pivoting
     double A[6][12];
     for (int r = 0; r < 6; ++r)
@@ -324,6 +385,23 @@ int quadric_inverse(int H, int W, QuadricInverse *qi)
     }
     for (int r = 0; r < 6; ++r)
         for (int c = 0; c < 6; ++c) qi->ginv[r * 6 + c] = A[r][c + 6];
+    return 0;
+}
+
+// The inverse for a pattern size, from the context's few latest sizes: summing the Gram matrix over the
+// pixels takes the host 0.2 ms at 128 x 128 and 15 ms at 1244 x 1024, more than the kernel on few patterns.
+int quadric_plan(hrebsd_ctx *ctx, int H, int W, QuadricInverse *qi)
+{
+    for (auto &q : ctx->quadrics)
+        if (q.H == H && q.W == W) {
+            memcpy(qi->ginv, q.ginv, sizeof qi->ginv);
+            return 0;
+        }
+    if (quadric_inverse(H, W, qi)) return -1;
+    if (ctx->quadrics.size() >= 8) ctx->quadrics.erase(ctx->quadrics.begin());
+    hr_quadric q{H, W, {}};
+    memcpy(q.ginv, qi->ginv, sizeof q.ginv);
+    ctx->quadrics.push_back(q);
     return 0;
 }
 
@@ -357,7 +435,8 @@ extern "C" int hrebsd_preprocess_batch(hrebsd_ctx *ctx, const float *in, int n, 
     if (st) return st;
     if (flat && (H > kMaxDim || W > kMaxDim)) return HREBSD_EINVAL;
     QuadricInverse qi;
-    if (flat && quadric_inverse(H, W, &qi)) return HREBSD_EINVAL;
+    if (flat && quadric_plan(ctx, H, W, &qi)) return HREBSD_EINVAL;
+    qi.mw = (unsigned)(((1ull << 32) + W - 1) / W);
     if (!flat)
         for (double &g : qi.ginv) g = 0.0;
     hr_prof_begin(ctx, hr_stream(stream));
