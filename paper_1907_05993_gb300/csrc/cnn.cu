@@ -62,22 +62,46 @@ __device__ __forceinline__ void store_input_pixel(bf16 *o, float r, float t)
     dst[1] = *reinterpret_cast<const uint4 *>(&v[4]);
 }
 
+// F: the block size where the rows of a block are read as one float2 / float4 (2, 4: pattern width and base
+// addresses on their boundary), 0: any.
+template <int F>
 __global__ void pack_patterns_kernel(const float *ref, const float *test, const int32_t *ref_idx, int B, int H, int W,
                                      bf16 *x)
 {
-    const int f = H / 64;
+    const int f = F ? F : H / 64;
     const float s = 1.0f / (float)(f * f);
     for (int b = blockIdx.y; b < B; b += gridDim.y)
         for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < 4096; p += gridDim.x * blockDim.x) {
             const int yy = p / 64, xx = p % 64;
-            const float *r = ref + (size_t)ref_idx[b] * H * W, *t = test + (size_t)b * H * W;
+            const size_t o0 = (size_t)(yy * f) * W + xx * f;
+            const float *r = ref + (size_t)ref_idx[b] * H * W + o0, *t = test + (size_t)b * H * W + o0;
             float sr = 0.0f, st = 0.0f;
-            for (int dy = 0; dy < f; ++dy)
-                for (int dx = 0; dx < f; ++dx) {
-                    const size_t o = (size_t)(yy * f + dy) * W + xx * f + dx;
-                    sr += r[o];
-                    st += t[o];
+            if constexpr (F == 0) {
+                for (int dy = 0; dy < f; ++dy)
+                    for (int dx = 0; dx < f; ++dx) {
+                        sr += r[(size_t)dy * W + dx];
+                        st += t[(size_t)dy * W + dx];
+                    }
+            } else {   // all rows first, then the sums in the same order
+                float rv[F][F], tv[F][F];
+#pragma unroll
+                for (int dy = 0; dy < F; ++dy) {
+                    if constexpr (F == 4) {
+                        *reinterpret_cast<float4 *>(tv[dy]) = __ldg(reinterpret_cast<const float4 *>(t + (size_t)dy * W));
+                        *reinterpret_cast<float4 *>(rv[dy]) = __ldg(reinterpret_cast<const float4 *>(r + (size_t)dy * W));
+                    } else {
+                        *reinterpret_cast<float2 *>(tv[dy]) = __ldg(reinterpret_cast<const float2 *>(t + (size_t)dy * W));
+                        *reinterpret_cast<float2 *>(rv[dy]) = __ldg(reinterpret_cast<const float2 *>(r + (size_t)dy * W));
+                    }
                 }
+#pragma unroll
+                for (int dy = 0; dy < F; ++dy)
+#pragma unroll
+                    for (int dx = 0; dx < F; ++dx) {
+                        sr += rv[dy][dx];
+                        st += tv[dy][dx];
+                    }
+            }
             store_input_pixel(x + ((size_t)b * 4096 + p) * 16, sr * s, st * s);
         }
 }
@@ -94,7 +118,7 @@ __global__ void pack_nchw_kernel(const bf16 *in, int B, bf16 *x)
 
 // 2x2 max-pool of NHWC BF16 (stride xs, offset xo, C channels, C and xs, xo
 // multiples of 8) -> dense [N][h/2][w/2][C] plus the argmax (0..3, first
-// maximum in row-major order of the 2x2 window).  One thread per 8 channels.
+// maximum in row-major order of the 2x2 window; arg null: not wanted).  One thread per 8 channels.
 __global__ void maxpool_kernel(const bf16 *x, int xs, int xo, int C, int N, int H, int W, bf16 *y, uint8_t *arg)
 {
     const int h = H / 2, w = W / 2, C8 = C / 8, per = h * w * C8;
@@ -127,25 +151,45 @@ __global__ void maxpool_kernel(const bf16 *x, int xs, int xo, int C, int N, int 
             }
             const size_t o = ((size_t)n * h * w + q) * C + c8 * 8;
             *reinterpret_cast<uint4 *>(y + o) = out;
-            *reinterpret_cast<uint2 *>(arg + o) = *reinterpret_cast<const uint2 *>(am);
+            if (arg) *reinterpret_cast<uint2 *>(arg + o) = *reinterpret_cast<const uint2 *>(am);
         }
 }
 
-// d_in[p][c] (FP32, dense [N][H][W][C]) = routed dy from the pool + skip gradient (stride ss, offset so).
-__global__ void maxpool_bwd_kernel(const float *dy, const uint8_t *arg, int C, int N, int H, int W, const float *skip,
-                                   int ss, int so, float *dx)
+// d_in[p][c] (FP32, dense [N][H][W][C]) = routed dy from the pool + skip gradient (stride ss, offset so).  One
+// thread per pooled pixel and 8 channels writes the window's four pixels (C, ss and so multiples of 8): the
+// index arithmetic and the pooled gradient once for 32 outputs.  The three levels of 256 pairs together about
+// 60 us (179 with one output per thread).
+__global__ void __launch_bounds__(256) maxpool_bwd_kernel(const float *dy, const uint8_t *arg, int C, int N, int H, int W,
+                                                          const float *skip, int ss, int so, float *dx)
 {
-    const size_t total = (size_t)N * H * W * C;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const size_t q = i / C;
-        const int xx = (int)(q % W), yy = (int)((q / W) % H), n = (int)(q / ((size_t)W * H));
-        const size_t pi = ((size_t)(n * (H / 2) + yy / 2) * (W / 2) + xx / 2) * C + c;
-        const int k = (yy & 1) * 2 + (xx & 1);
-        float v = arg[pi] == k ? dy[pi] : 0.0f;
-        if (skip) v += skip[q * ss + so + c];
-        dx[i] = v;
-    }
+    const int h = H / 2, w = W / 2, C8 = C / 8, per = h * w * C8;
+    for (int n = blockIdx.y; n < N; n += gridDim.y)
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < per; i += gridDim.x * blockDim.x) {
+            const int c8 = i % C8, q = i / C8, xx = q % w, yy = q / w;
+            const size_t o = ((size_t)n * h * w + q) * C + c8 * 8;
+            const uint2 av = *reinterpret_cast<const uint2 *>(arg + o);
+            const float4 d0 = *reinterpret_cast<const float4 *>(dy + o), d1 = *reinterpret_cast<const float4 *>(dy + o + 4);
+            const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+            float4 s0[4], s1[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const size_t p = ((size_t)n * H + 2 * yy + k / 2) * W + 2 * xx + k % 2;
+                const float *sp = skip + p * ss + so + c8 * 8;
+                s0[k] = skip ? *reinterpret_cast<const float4 *>(sp) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                s1[k] = skip ? *reinterpret_cast<const float4 *>(sp + 4) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const size_t p = ((size_t)n * H + 2 * yy + k / 2) * W + 2 * xx + k % 2;
+                float v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    v[e] = (((e < 4 ? av.x : av.y) >> (8 * (e & 3))) & 255u) == (unsigned)k ? d[e] : 0.0f;
+                float *dst = dx + p * C + c8 * 8;
+                *reinterpret_cast<float4 *>(dst) = make_float4(v[0] + s0[k].x, v[1] + s0[k].y, v[2] + s0[k].z, v[3] + s0[k].w);
+                *reinterpret_cast<float4 *>(dst + 4) = make_float4(v[4] + s1[k].x, v[5] + s1[k].y, v[6] + s1[k].z, v[7] + s1[k].w);
+            }
+        }
 }
 
 // Nearest up-sampling x2 of dense [N][h][w][C] BF16 into y (stride ys, offset
@@ -161,19 +205,29 @@ __global__ void up2_kernel(const bf16 *x, int C, int N, int h, int w, bf16 *y, i
         }
 }
 
-// Adjoint of up2: dx[N][h][w][C] = sum of the 4 children of dy (stride ys, offset yo).
-__global__ void up2_bwd_kernel(const float *dy, int ys, int yo, int C, int N, int h, int w, float *dx)
+// Adjoint of up2: dx[N][h][w][C] = sum of the 4 children of dy (stride ys, offset yo), 4 channels per thread
+// (C, ys and yo multiples of 4).
+__global__ void __launch_bounds__(256) up2_bwd_kernel(const float *dy, int ys, int yo, int C, int N, int h, int w, float *dx)
 {
-    const int W = 2 * w;
-    const size_t total = (size_t)N * h * w * C;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const size_t q = i / C;
-        const int xx = (int)(q % w), yy = (int)((q / w) % h), n = (int)(q / ((size_t)w * h));
-        float s = 0.0f;
-        for (int k = 0; k < 4; ++k) s += dy[((size_t)(n * 2 * h + 2 * yy + k / 2) * W + 2 * xx + k % 2) * ys + yo + c];
-        dx[i] = s;
-    }
+    const int W = 2 * w, C4 = C / 4, per = h * w * C4;
+    for (int n = blockIdx.y; n < N; n += gridDim.y)
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < per; i += gridDim.x * blockDim.x) {
+            const int c4 = i % C4, q = i / C4, xx = q % w, yy = q / w;
+            float4 v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                v[k] = *reinterpret_cast<const float4 *>(
+                    dy + (((size_t)n * 2 * h + 2 * yy + k / 2) * W + 2 * xx + k % 2) * ys + yo + c4 * 4);
+            float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                s.x += v[k].x;
+                s.y += v[k].y;
+                s.z += v[k].z;
+                s.w += v[k].w;
+            }
+            *reinterpret_cast<float4 *>(dx + ((size_t)n * h * w + q) * C + c4 * 4) = s;
+        }
 }
 
 // dpre (BF16 dense [P][C]) = dpost (FP32, stride ds, offset do) * (out > 0), out BF16 (stride os, offset oo).
@@ -322,20 +376,31 @@ __global__ void head_bwd_kernel(const float *dout, const bf16 *d1, const bf16 *w
 {
     __shared__ float red[256][HEAD_COUT * (HEAD_CIN + 1)];
     float acc[HEAD_COUT * (HEAD_CIN + 1)];
+#pragma unroll
     for (int k = 0; k < HEAD_COUT * (HEAD_CIN + 1); ++k) acc[k] = 0.0f;
     const size_t total = (size_t)N * 4096;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const size_t b = i / 4096, p = i % 4096;
         const float g0 = dout[b * 8192 + p], g1 = dout[b * 8192 + 4096 + p];
+        uint4 in[2];   // the pixel's 16 channels
+        in[0] = reinterpret_cast<const uint4 *>(d1 + i * HEAD_CIN)[0];
+        in[1] = reinterpret_cast<const uint4 *>(d1 + i * HEAD_CIN)[1];
+        const bf16 *e = reinterpret_cast<const bf16 *>(in);
+        float dd[HEAD_CIN];
+#pragma unroll
         for (int c = 0; c < HEAD_CIN; ++c) {
-            const float v = __bfloat162float(d1[i * HEAD_CIN + c]);
-            dd1[i * HEAD_CIN + c] = __bfloat162float(w[c]) * g0 + __bfloat162float(w[HEAD_CIN + c]) * g1;
+            const float v = __bfloat162float(e[c]);
+            dd[c] = __bfloat162float(w[c]) * g0 + __bfloat162float(w[HEAD_CIN + c]) * g1;
             acc[c] = fmaf(g0, v, acc[c]);
             acc[HEAD_CIN + 1 + c] = fmaf(g1, v, acc[HEAD_CIN + 1 + c]);
         }
+#pragma unroll
+        for (int c = 0; c < HEAD_CIN; c += 4)
+            *reinterpret_cast<float4 *>(dd1 + i * HEAD_CIN + c) = make_float4(dd[c], dd[c + 1], dd[c + 2], dd[c + 3]);
         acc[HEAD_CIN] += g0;
         acc[2 * HEAD_CIN + 1] += g1;
     }
+#pragma unroll
     for (int k = 0; k < HEAD_COUT * (HEAD_CIN + 1); ++k) red[threadIdx.x][k] = acc[k];
     __syncthreads();
     if (threadIdx.x < HEAD_COUT * (HEAD_CIN + 1)) {
@@ -592,8 +657,19 @@ int launch_halo_t(hrebsd_ctx *ctx, const ConvArgs &a, cudaStream_t st)
 
 // Halo tiles by TMA into tcgen05 MMAs (forward convolutions with BF16 output and
 // the tiled weight copy).  Returns 1 when the shape is not covered.
+// What the epilogue of a convolution makes of its output besides (or, with `only`, instead of) storing it;
+// `done` tells whether the kernel that ran did so (the tcgen05 forward kernel does).
+struct Fuse {
+    bf16 *yu = nullptr;          // up-sampled x2, channel stride yus, offset 0
+    int yus = 0;
+    const bf16 *hw = nullptr;    // 1x1 head
+    const float *hb = nullptr;
+    float *hout = nullptr;
+    bool only = false, done = false;
+};
+
 template <int RES>
-int launch_tma_t(hrebsd_ctx *ctx, const ConvArgs &a, const bf16 *wt, cudaStream_t st)
+int launch_tma_t(hrebsd_ctx *ctx, const ConvArgs &a, const bf16 *wt, Fuse *fz, cudaStream_t st)
 {
     using G = TmaGeom<RES>;
     constexpr int BN = G::BN;
@@ -603,6 +679,13 @@ int launch_tma_t(hrebsd_ctx *ctx, const ConvArgs &a, const bf16 *wt, cudaStream_
     t.bias = a.bias;
     t.y = a.y_fp32 ? nullptr : reinterpret_cast<bf16 *>(a.y);
     t.yf = a.y_fp32 ? reinterpret_cast<float *>(a.y) : nullptr;
+    t.yu = fz ? fz->yu : nullptr;
+    t.yus = fz ? fz->yus : 0;
+    t.yuo = 0;
+    t.hw = fz ? fz->hw : nullptr;
+    t.hb = fz ? fz->hb : nullptr;
+    t.hout = fz ? fz->hout : nullptr;
+    if (fz && fz->only) t.y = nullptr;
     t.ys = a.ys;
     t.yo = a.yo;
     t.relu = a.relu;
@@ -655,18 +738,20 @@ int launch_tma_t(hrebsd_ctx *ctx, const ConvArgs &a, const bf16 *wt, cudaStream_
     if (by_smem < per_sm) per_sm = by_smem;
     const long long grid = tiles < (long long)ctx->num_sms * per_sm ? tiles : (long long)ctx->num_sms * per_sm;
     conv3x3_tma_tc_kernel<RES><<<(unsigned)grid, kTmaConvThreads, smem, st>>>(tm, t, ctx->d_err);
-    return cudaGetLastError() == cudaSuccess ? HREBSD_OK : HREBSD_ECUDA;
+    if (cudaGetLastError() != cudaSuccess) return HREBSD_ECUDA;
+    if (fz) fz->done = true;
+    return HREBSD_OK;
 }
 
-int launch_tma_conv(hrebsd_ctx *ctx, const ConvArgs &a, const bf16 *wt, cudaStream_t st)
+int launch_tma_conv(hrebsd_ctx *ctx, const ConvArgs &a, const bf16 *wt, Fuse *fz, cudaStream_t st)
 {
     if (!wt || !ctx->cnn_tc || a.H != a.W || a.N < 1 || a.cin % 16) return 1;
     if (a.xs % 8 || a.xo % 8 || a.ys % 8 || a.yo % 8) return 1;
     switch (a.H) {
-    case 64: return launch_tma_t<64>(ctx, a, wt, st);
-    case 32: return launch_tma_t<32>(ctx, a, wt, st);
-    case 16: return launch_tma_t<16>(ctx, a, wt, st);
-    case 8: return launch_tma_t<8>(ctx, a, wt, st);
+    case 64: return launch_tma_t<64>(ctx, a, wt, fz, st);
+    case 32: return launch_tma_t<32>(ctx, a, wt, fz, st);
+    case 16: return launch_tma_t<16>(ctx, a, wt, fz, st);
+    case 8: return launch_tma_t<8>(ctx, a, wt, fz, st);
     default: return 1;
     }
 }
@@ -693,7 +778,7 @@ int launch_halo_conv(hrebsd_ctx *ctx, const ConvArgs &a, cudaStream_t st)
 }
 
 int conv(hrebsd_ctx *ctx, const bf16 *x, int xs, int xo, int cin, const bf16 *w, const float *bias, int cout, void *y,
-         int ys, int yo, int y_fp32, int relu, int N, int res, cudaStream_t st, const bf16 *wt = nullptr)
+         int ys, int yo, int y_fp32, int relu, int N, int res, cudaStream_t st, const bf16 *wt = nullptr, Fuse *fz = nullptr)
 {
     ConvArgs a;
     a.x = x;
@@ -713,7 +798,7 @@ int conv(hrebsd_ctx *ctx, const bf16 *x, int xs, int xo, int cin, const bf16 *w,
     a.W = res;
     const int P = N * res * res;
     hr_prof_begin(ctx, st);
-    int e = launch_tma_conv(ctx, a, wt, st);
+    int e = launch_tma_conv(ctx, a, wt, fz, st);
     if (e == 1) e = launch_halo_conv(ctx, a, st);
     if (e == 1) {   // no halo variant for this shape: pipelined implicit GEMM
         // output-channel tile: the largest of 64, 32, 16 that divides cout
@@ -876,34 +961,50 @@ void layer_views(hr_cnn_net *n, View *in, View *out)
     out[13] = {n->act[13], 16, 0};
 }
 
-int forward(hrebsd_ctx *ctx, int B, cudaStream_t st)
+// out: the planar FP32 field.  train: keep what the backward pass reads (every activation, the pools' argmax);
+// otherwise the outputs that only the up-sampling or the head reads are not written (the epilogue makes the
+// up-sampled copy and the field).
+int forward(hrebsd_ctx *ctx, int B, float *result, bool train, cudaStream_t st)
 {
     hr_cnn_net *n = ctx->cnn;
     View in[NCONV], out[NCONV];
     layer_views(n, in, out);
     int e;
-    auto run = [&](int l) {
+    auto run = [&](int l, Fuse *fz = nullptr) {
         return conv(ctx, in[l].p, in[l].s, in[l].o, pad16(kLayers[l].cin), n->wf[l], n->W + n->b_off[l],
-                    kLayers[l].cout, out[l].p, out[l].s, out[l].o, 0, 1, B, kLayers[l].res, st, n->wt[l]);
+                    kLayers[l].cout, out[l].p, out[l].s, out[l].o, 0, 1, B, kLayers[l].res, st, n->wt[l], fz);
     };
     auto pool = [&](int k, const View &v, int C, int res) {
         maxpool_kernel<<<grid2(res * res / 4 * C / 8, B), 256, 0, st>>>(v.p, v.s, v.o, C, B, res, res, n->pool[k],
-                                                                       n->parg[k]);
+                                                                       train ? n->parg[k] : nullptr);
         return cudaGetLastError() == cudaSuccess ? (ctx->launches++, HREBSD_OK) : HREBSD_ECUDA;
     };
-    auto up = [&](const bf16 *src, int C, int res, bf16 *dst, int ds) {
-        up2_kernel<<<grid2(res * res * 4 * C / 8, B), 256, 0, st>>>(src, C, B, res, res, dst, ds, 0);
+    auto run_up = [&](int l, bf16 *dst, int ds) {   // layer l and its up-sampled copy
+        Fuse fz;
+        fz.yu = dst;
+        fz.yus = ds;
+        fz.only = !train;
+        const int e2 = run(l, &fz);
+        if (e2 || fz.done) return e2;
+        const int C = kLayers[l].cout, res = kLayers[l].res;
+        up2_kernel<<<grid2(res * res * 4 * C / 8, B), 256, 0, st>>>(out[l].p, C, B, res, res, dst, ds, 0);
         return cudaGetLastError() == cudaSuccess ? (ctx->launches++, HREBSD_OK) : HREBSD_ECUDA;
     };
     if ((e = run(0)) || (e = run(1)) || (e = pool(0, out[1], 16, 64))) return e;
     if ((e = run(2)) || (e = run(3)) || (e = pool(1, out[3], 32, 32))) return e;
     if ((e = run(4)) || (e = run(5)) || (e = pool(2, out[5], 64, 16))) return e;
-    if ((e = run(6)) || (e = run(7)) || (e = up(n->act[7], 128, 8, n->cat3, 192))) return e;
-    if ((e = run(8)) || (e = run(9)) || (e = up(n->act[9], 64, 16, n->cat2, 96))) return e;
-    if ((e = run(10)) || (e = run(11)) || (e = up(n->act[11], 32, 32, n->cat1, 48))) return e;
-    if ((e = run(12)) || (e = run(13))) return e;
+    if ((e = run(6)) || (e = run_up(7, n->cat3, 192))) return e;
+    if ((e = run(8)) || (e = run_up(9, n->cat2, 96))) return e;
+    if ((e = run(10)) || (e = run_up(11, n->cat1, 48))) return e;
+    Fuse fz;
+    fz.hw = n->wf[NCONV];
+    fz.hb = n->W + n->b_off[NCONV];
+    fz.hout = result;
+    fz.only = !train;
+    if ((e = run(12)) || (e = run(13, &fz))) return e;
+    if (fz.done) return HREBSD_OK;
     hr_prof_begin(ctx, st);
-    head_fwd_kernel<<<grid2(4096, B), 256, 0, st>>>(n->act[13], n->wf[NCONV], n->W + n->b_off[NCONV], B, n->out);
+    head_fwd_kernel<<<grid2(4096, B), 256, 0, st>>>(n->act[13], n->wf[NCONV], n->W + n->b_off[NCONV], B, result);
     hr_prof_end(ctx, PROF_CNN, st);
     HR_LAUNCHED(ctx);
     return HREBSD_OK;
@@ -958,12 +1059,12 @@ int backward(hrebsd_ctx *ctx, int B, cudaStream_t st)
     HR_LAUNCHED(ctx);
     const size_t p64 = (size_t)B * 4096, p32 = p64 / 4, p16 = p64 / 16;
     auto ub = [&](const float *src, int ss, int C, int res, float *dst) {   // res: coarse size
-        up2_bwd_kernel<<<grid_for(ctx, (size_t)B * res * res * C), 256, 0, st>>>(src, ss, 0, C, B, res, res, dst);
+        up2_bwd_kernel<<<grid2(res * res * C / 4, B), 256, 0, st>>>(src, ss, 0, C, B, res, res, dst);
         return cudaGetLastError() == cudaSuccess ? (ctx->launches++, HREBSD_OK) : HREBSD_ECUDA;
     };
     auto pb = [&](int k, const float *dp, int C, int res, const float *skip, int ss, int so, float *dst) {
-        maxpool_bwd_kernel<<<grid_for(ctx, (size_t)B * res * res * C), 256, 0, st>>>(dp, n->parg[k], C, B, res, res,
-                                                                                    skip, ss, so, dst);
+        maxpool_bwd_kernel<<<grid2(res * res / 4 * C / 8, B), 256, 0, st>>>(dp, n->parg[k], C, B, res, res, skip, ss, so,
+                                                                           dst);
         return cudaGetLastError() == cudaSuccess ? (ctx->launches++, HREBSD_OK) : HREBSD_ECUDA;
     };
     // decoder level 1 (64x64)
@@ -1155,10 +1256,7 @@ extern "C" int hrebsd_cnn_load(hrebsd_ctx *ctx, const char *path)
 
 static int infer_common(hrebsd_ctx *ctx, int B, float *field, cudaStream_t st)
 {
-    int e = forward(ctx, B, st);
-    if (e) return e;
-    HR_CHECK(cudaMemcpyAsync(field, ctx->cnn->out, (size_t)B * 8192 * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    return HREBSD_OK;
+    return forward(ctx, B, field, false, st);
 }
 
 extern "C" int hrebsd_cnn_infer(hrebsd_ctx *ctx, const uint16_t *x_bf16, int B, float *field64, void *stream)
@@ -1185,7 +1283,10 @@ extern "C" int hrebsd_cnn_infer_patterns(hrebsd_ctx *ctx, const float *ref, cons
     int e = hr_set_device(ctx);
     if (e || (e = ensure_acts(ctx, B))) return e;
     cudaStream_t st = hr_stream(stream);
-    pack_patterns_kernel<<<grid2(4096, B), 256, 0, st>>>(ref, test, ref_idx, B, H, W, ctx->cnn->x);
+    const int f = H / 64;
+    const bool aligned = ((reinterpret_cast<uintptr_t>(ref) | reinterpret_cast<uintptr_t>(test)) % (4 * f)) == 0;
+    auto pack = f == 4 && aligned ? pack_patterns_kernel<4> : f == 2 && aligned ? pack_patterns_kernel<2> : pack_patterns_kernel<0>;
+    pack<<<grid2(4096, B), 256, 0, st>>>(ref, test, ref_idx, B, H, W, ctx->cnn->x);
     HR_LAUNCHED(ctx);
     return infer_common(ctx, B, field64, st);
 }
@@ -1200,7 +1301,7 @@ extern "C" int hrebsd_cnn_train_step(hrebsd_ctx *ctx, const uint16_t *x_bf16, co
     cudaStream_t st = hr_stream(stream);
     pack_nchw_kernel<<<grid2(4096, B), 256, 0, st>>>(reinterpret_cast<const bf16 *>(x_bf16), B, n->x);
     HR_LAUNCHED(ctx);
-    if ((e = forward(ctx, B, st))) return e;
+    if ((e = forward(ctx, B, n->out, true, st))) return e;
     HR_CHECK(cudaMemsetAsync(n->loss, 0, sizeof(float), st));
     HR_CHECK(cudaMemsetAsync(n->G, 0, n->n_params * sizeof(float), st));
     mse_kernel<<<grid_for(ctx, (size_t)B * 8192), 256, 0, st>>>(n->out, target, (size_t)B * 8192, n->dout, n->loss);

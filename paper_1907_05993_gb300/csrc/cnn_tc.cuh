@@ -55,7 +55,13 @@ struct TmaGeom {
 struct TmaConvArgs {
     const bf16 *wt;      // [cout / BN][cin / 16][2][9][BN][8]
     const float *bias;   // [cout] or null
-    bf16 *y;             // output (NHWC, channel stride ys, offset yo), or null when yf is set
+    bf16 *y;             // output (NHWC, channel stride ys, offset yo), or null when yf is set or the layer after
+                         // this one only reads what the epilogue makes of it (yu, head)
+    bf16 *yu;            // the output up-sampled x2 (nearest; NHWC, channel stride yus, offset yuo), or null
+    const bf16 *hw;      // 1x1 head on the output (cout = BN = 16): weights [2][16], bias [2] and the planar FP32
+    const float *hb;     // result [N][2][RES][RES], or null
+    float *hout;
+    int yus, yuo;
     float *yf;           // FP32 output in the same layout (the input gradients), or null
     int ys, yo, relu;
     int cin, cout, N;
@@ -106,7 +112,7 @@ __global__ void __launch_bounds__(kTmaConvThreads, 1)
     __shared__ __align__(8) uint64_t full[MAXST], empty[MAXST], accf[2], acce[2], drain;
     __shared__ uint32_t tmem_base;
     __shared__ int abort_s;
-    __shared__ float bias_s[256];
+    __shared__ float bias_s[256], head_s[34];
     // swizzled boxes need 1024-byte aligned buffers: the host adds 1 KB of slack
     unsigned char *tc_smem = tc_smem_raw + ((1024u - (hr_tma::smem_u32(tc_smem_raw) & 1023u)) & 1023u);
     volatile int *abort = &abort_s;
@@ -129,6 +135,7 @@ __global__ void __launch_bounds__(kTmaConvThreads, 1)
         hr_tma::fence_mbar_init();
     }
     for (int i = tid; i < a.cout; i += blockDim.x) bias_s[i] = a.bias ? a.bias[i] : 0.0f;
+    if (a.hout && tid < 34) head_s[tid] = tid < 32 ? __bfloat162float(a.hw[tid]) : a.hb[tid - 32];
     if (warp == 1) hr_tc::tmem_alloc(&tmem_base, (uint32_t)G::TMEM);
     hr_tc::fence_before_sync();
     __syncthreads();
@@ -239,20 +246,43 @@ __global__ void __launch_bounds__(kTmaConvThreads, 1)
                         dst[c0 / 4] = o4;
                     }
                 } else if (prel[j] >= 0 && T.n0 + pnl[j] < a.N) {
-                    uint4 *dst = reinterpret_cast<uint4 *>(a.y + (pbase + prel[j]) * a.ys + a.yo + o0);
+                    __align__(16) __nv_bfloat162 o2[BN / 2];
 #pragma unroll
-                    for (int c0 = 0; c0 < BN; c0 += 8) {
-                        __align__(16) __nv_bfloat162 o2[4];
-#pragma unroll
-                        for (int k = 0; k < 8; k += 2) {
-                            float v0 = v[c0 + k] + bias_s[o0 + c0 + k], v1 = v[c0 + k + 1] + bias_s[o0 + c0 + k + 1];
-                            if (a.relu) {
-                                v0 = fmaxf(v0, 0.0f);
-                                v1 = fmaxf(v1, 0.0f);
-                            }
-                            o2[k / 2] = __floats2bfloat162_rn(v0, v1);
+                    for (int k = 0; k < BN; k += 2) {
+                        float v0 = v[k] + bias_s[o0 + k], v1 = v[k + 1] + bias_s[o0 + k + 1];
+                        if (a.relu) {
+                            v0 = fmaxf(v0, 0.0f);
+                            v1 = fmaxf(v1, 0.0f);
                         }
-                        dst[c0 / 8] = *reinterpret_cast<const uint4 *>(o2);
+                        o2[k / 2] = __floats2bfloat162_rn(v0, v1);
+                    }
+                    const uint4 *o4 = reinterpret_cast<const uint4 *>(o2);
+                    if (a.y) {
+                        uint4 *dst = reinterpret_cast<uint4 *>(a.y + (pbase + prel[j]) * a.ys + a.yo + o0);
+#pragma unroll
+                        for (int k = 0; k < BN / 8; ++k) dst[k] = o4[k];
+                    }
+                    const int y = T.y0 + prel[j] / RES % RES, x = prel[j] % RES, img = T.n0 + pnl[j];
+                    if (a.yu) {
+                        bf16 *up = a.yu + (((size_t)img * 2 * RES + 2 * y) * 2 * RES + 2 * x) * a.yus + a.yuo + o0;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            uint4 *dst = reinterpret_cast<uint4 *>(up + (size_t)((c >> 1) * 2 * RES + (c & 1)) * a.yus);
+#pragma unroll
+                            for (int k = 0; k < BN / 8; ++k) dst[k] = o4[k];
+                        }
+                    }
+                    if (BN == 16 && a.hout) {   // on the rounded activations, as from memory
+                        float a0 = head_s[32], a1 = head_s[33];
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            const float t = k & 1 ? __high2float(o2[k / 2]) : __low2float(o2[k / 2]);
+                            a0 = fmaf(head_s[k], t, a0);
+                            a1 = fmaf(head_s[16 + k], t, a1);
+                        }
+                        float *h = a.hout + (size_t)img * 2 * RES * RES + y * RES + x;
+                        h[0] = a0;
+                        h[RES * RES] = a1;
                     }
                 }
             }
