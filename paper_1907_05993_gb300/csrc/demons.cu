@@ -827,9 +827,11 @@ __global__ void __launch_bounds__(NT_, MINB) demons_iter_tma_kernel(const __grid
     if (tid == 0 && prev_pair >= 0) write_partial();
 }
 
+
 #include "demons_strip.cuh"
 #include "demons_level.cuh"
 #include "demons_cluster.cuh"
+#include "demons_wide.cuh"
 
 struct CtrlArgs {
     const float *part;       // [B][tiles]
@@ -1386,6 +1388,87 @@ int launch_cluster(hrebsd_ctx *ctx, const clu::ClusterArgs &a, const ClusterPlan
     return HREBSD_OK;
 }
 
+// The sweep over strips and bands: threads per CTA, strips, bands.  A band's 12 extra rows and a strip's halo
+// columns are recomputed; a wave of CTAs takes about as long half full as full.  Estimated SM cycles as
+// shape_cycles, fitted to 18 sizes, 23 x 25 to 1244 x 1024 (within ~20 %; the chosen split was the fastest of
+// all, or within 8 % of it, at each).  NT = 0: none.
+struct WidePlan {
+    int NT = 0;
+    wide::WideArgs w{};
+    float cycles = 0.0f;
+};
+WidePlan plan_wide(const hrebsd_ctx *ctx, int B, int h, int w, bool regroup)
+{
+    WidePlan best;
+    for (int NT = 128; NT <= 256; NT *= 2) {
+        wide::WideArgs a{};
+        a.strips = (w + NT - 16) / (NT - 15);
+        a.sw = (w + a.strips - 1) / a.strips;
+        if (w - (a.strips - 1) * a.sw < 2 * wide::RAD) continue;   // (a strip's halo ends within the next one)
+        const long long cap = (long long)ctx->num_sms * (512 / NT);
+        for (int bands = 1; bands == 1 || (bands <= 64 && h / bands >= 16); ++bands) {
+            a.bh = (h + bands - 1) / bands;
+            a.bands = (h + a.bh - 1) / a.bh;
+            const long long items = (long long)B * a.strips * a.bands;
+            const int steps = (a.bh + (a.bands > 1 ? 18 : 12)) / 7;
+            const float waves = items <= cap ? 0.75f + 0.25f * (float)items / (float)cap : (float)((items + cap - 1) / cap);
+            const float cycles = waves * (26000.0f + 5900.0f * (float)steps);
+            if (!best.NT || cycles < best.cycles) {
+                best.NT = NT;
+                best.w = a;
+                best.cycles = cycles;
+            }
+        }
+    }
+    if (regroup) best.cycles += 6000.0f + 0.82f * (float)B * (float)(h * w) / (float)ctx->num_sms;
+    return best;
+}
+
+template <int NT, bool IN_S, bool TEX>
+int launch_wide_t(hrebsd_ctx *ctx, const IterArgs &a, const wide::WideArgs &wa, int max_items, cudaStream_t st)
+{
+    using G = wide::Geo<NT>;
+    static int configured_dev = -1;
+    static int occ = 0;
+    auto k = wide::demons_wide_kernel<NT, IN_S, TEX>;
+    if (configured_dev != ctx->device) {
+        HR_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::BYTES));
+        HR_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, NT, G::BYTES));
+        if (occ < 1) occ = 1;
+        configured_dev = ctx->device;
+    }
+    int grid = ctx->num_sms * occ;
+    if (grid > max_items) grid = max_items;
+    if (grid < 1) grid = 1;
+    hr_prof_begin(ctx, st);
+    k<<<grid, NT, G::BYTES, st>>>(a, wa);
+    hr_prof_end(ctx, PROF_ITER, st);
+    HR_LAUNCHED(ctx);
+    return HREBSD_OK;
+}
+
+template <int NT>
+int launch_wide_nt(hrebsd_ctx *ctx, const IterArgs &a, const wide::WideArgs &wa, int items, cudaStream_t st)
+{
+    if (a.mtex) return a.in_is_s ? launch_wide_t<NT, true, true>(ctx, a, wa, items, st) : launch_wide_t<NT, false, true>(ctx, a, wa, items, st);
+    return a.in_is_s ? launch_wide_t<NT, true, false>(ctx, a, wa, items, st) : launch_wide_t<NT, false, false>(ctx, a, wa, items, st);
+}
+
+// One iteration over the active pairs; a.tiles (and tiles_x) are the tile shape's where wa.dbuf is set, and
+// its partials are then formed from the stored d.
+int launch_wide(hrebsd_ctx *ctx, const WidePlan &p, const IterArgs &a, int tx, int ty, int nt, bool plain, int B, cudaStream_t st)
+{
+    const int items = B * p.w.strips * p.w.bands;
+    const int e = p.NT == 256 ? launch_wide_nt<256>(ctx, a, p.w, items, st) : launch_wide_nt<128>(ctx, a, p.w, items, st);
+    if (e || !p.w.dbuf) return e;
+    const long long groups = (long long)B * a.tiles, cap = (long long)ctx->num_sms * (2048 / nt);
+    hr_prof_begin(ctx, st);
+    wide::ssd_group_kernel<<<(unsigned)(groups < cap ? groups : cap), nt, 0, st>>>(a, p.w.dbuf, tx, ty, plain);
+    hr_prof_end(ctx, PROF_CTRL, st);
+    HR_LAUNCHED(ctx);
+    return HREBSD_OK;
+}
+
 // Pairs the loop form keeps resident at once (one CTA each) at a level w pixels wide.
 template <int NT>
 int strip_capacity_t(hrebsd_ctx *ctx)
@@ -1477,6 +1560,7 @@ int hr_graph_run(hrebsd_ctx *ctx, const hr_graph_key &key, cudaStream_t st, Emit
 // height, a stream that is being captured (no allocation or synchronisation inside a capture), or an
 // array that could not be allocated.  Growing an array synchronises the device (the old one may be in
 // use) and drops the cached graphs (their launches name the old texture).
+constexpr size_t kMaxTextures = 12;   // level widths with an array
 int hr_ref_texture(hrebsd_ctx *ctx, const float *ref, int R, int h, int w, cudaStream_t st, unsigned long long *tex)
 {
     *tex = 0;
@@ -1491,12 +1575,14 @@ int hr_ref_texture(hrebsd_ctx *ctx, const float *ref, int R, int h, int w, cudaS
         HR_CHECK(cudaDeviceGetAttribute(&mh, cudaDevAttrMaxTexture2DGatherHeight, ctx->device));
         HR_CHECK(cudaDeviceGetAttribute(&mw, cudaDevAttrMaxTexture2DGatherWidth, ctx->device));
         ctx->tex_max_rows = mw >= 256 && mh > 0 ? mh : -1;
+        ctx->tex_max_cols = mw;
     }
     const long long rows = (long long)R * h;
-    if (ctx->tex_max_rows < 0 || rows > ctx->tex_max_rows || w > 256) return HREBSD_OK;
+    if (ctx->tex_max_rows < 0 || rows > ctx->tex_max_rows || w > ctx->tex_max_cols) return HREBSD_OK;
     size_t mi = ctx->mtex.size();
     for (size_t i = 0; i < ctx->mtex.size(); ++i)
         if (ctx->mtex[i].w == w) mi = i;
+    if (mi == kMaxTextures) return HREBSD_OK;   // (bounded: further widths go without)
     if (mi == ctx->mtex.size() || ctx->mtex[mi].rows < rows) {
         long long cap_rows = rows > 8LL * h ? rows : 8LL * h;   // room for 8 references from the start
         if (mi < ctx->mtex.size()) {
@@ -1660,7 +1746,8 @@ int dispatch_finalize(hrebsd_ctx *ctx, int rad, bool planar, const float2 *u0, c
 
 enum { WS_TPYR = 0, WS_RPYR, WS_U0, WS_S0, WS_S1, WS_UOUT, WS_PART, WS_HIST, WS_LIST, WS_COUNT };
 
-// Register B pairs (all buffers already offset to this chunk).
+constexpr int WS_DBUF = 22;   // d of every pixel, for the regrouped SSD of the strip-and-band sweep
+
 // Bytes of each workspace slot for B pairs (WS_* order).
 void slot_bytes(int R, int B, int H, int W, const hrebsd_demons_params *p, size_t *bytes)
 {
@@ -1777,26 +1864,45 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
         const bool use_tma = !use_level && !use_strip && rad > 0 && !ctx->no_tma && cap > 1 &&
                              encode_maps(rad, var, (const float2 *)s0, (const float2 *)s1, (const float2 *)u0, tl[l],
                                          B, h, w, tmS, &tmF);
-        // the whole level in the shared memory of a cluster per pair, where that is estimated to be faster
-        // and the caller did not pin another shape
+        // where the caller did not pin a shape: the whole level in the shared memory of a cluster per pair, or
+        // the sweep over strips and bands in place of the tiles, whichever is estimated to be the fastest
         ClusterPlan plan;
         clu::ClusterArgs ca;
+        WidePlan wp;
+        const int tile_tx = use_tma ? kVarTX[var] : TX, tile_ty = use_tma ? kVarTY[var] : TY;
         if (rad == clu::RAD && cap >= 1 && !ctx->no_tma && !hr_pinned_variant(ctx, h, w)) {
             const LevelShape shape{var, use_level, use_strip, use_tma};
             // the rule can end the level before the cap: the SSD has to be summed as that shape sums it
             const bool regroup = p->stop_window > 0 && cap > p->stop_window;
             const bool tile = !use_level && !use_strip;
+            float limit = 0.9f * shape_cycles(ctx, shape, B, h, w);
+            // (the estimate for the plain-load tiles is up to 15 % low, that for the TMA-fed ones up to 25 % high;
+            // the sweep's is low, the cluster's high at narrow levels)
+            if (tile && !given && h >= 8 && w >= 8 && (long long)h * w < (1 << 24)) {
+                wp = plan_wide(ctx, B, h, w, regroup);
+                if (wp.NT && wp.cycles < (use_tma ? 0.89f : 1.17f) * limit) limit = fminf(limit, 1.2f * wp.cycles);
+                else wp.NT = 0;
+            }
             ca.group = !regroup ? clu::G_FREE : use_level ? clu::G_LEVEL : use_strip ? clu::G_STRIP : use_tma ? clu::G_TILE : clu::G_PLAIN;
-            ca.tx = !tile ? w : use_tma ? kVarTX[var] : TX;
-            ca.ty = !tile ? h : use_tma ? kVarTY[var] : TY;
+            ca.tx = tile ? tile_tx : w;
+            ca.ty = tile ? tile_ty : h;
             ca.nt = use_level ? lvl::NT : use_strip ? w : use_tma ? kVarNT[var] : kIterThreads;
             ca.tiles_x = (w + ca.tx - 1) / ca.tx;
             ca.tiles = ca.tiles_x * ((h + ca.ty - 1) / ca.ty);
             ca.tasks = ca.tiles * (ca.nt / 32);
             if (!regroup || ca.tasks <= clu::MAX_TASKS) {
                 if ((e = plan_cluster(ctx, B, h, w, ca.group, ca.tasks, &plan))) return e;
-                if (plan.C && plan.cycles > 0.9f * shape_cycles(ctx, shape, B, h, w)) plan.C = 0;
+                if (plan.C && plan.cycles > limit) plan.C = 0;
             }
+            if (plan.C) wp.NT = 0;
+            if (wp.NT && regroup) {
+                void *d = nullptr;
+                e = hr_ws(ctx, WS_DBUF, (size_t)B * H * W * 4, &d);
+                if (e == HREBSD_ENOMEM) wp.NT = 0;   // no room for d: the tiles do without
+                else if (e) return e;
+                wp.w.dbuf = (float *)d;
+            }
+            if (wp.NT && (e = hr_ref_texture(ctx, rl[l], R, h, w, st, &mtex))) return e;
         }
         // The launches of one level: list reset, cap x (iteration, control) -- or, in the loop
         // form, iteration 0 and its control, then one launch for the rest --, finalize,
@@ -1873,8 +1979,9 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
             for (int k = 0; k < (use_loop ? 1 : cap); ++k) {
                 const bool tma_k = !use_strip && use_tma && (k > 0 || rad == 3);
                 const int tx = tma_k ? kVarTX[var] : TX, ty = tma_k ? kVarTY[var] : TY;
-                const int tiles_x = use_strip ? 1 : (w + tx - 1) / tx;
-                const int tiles = use_strip ? 1 : tiles_x * ((h + ty - 1) / ty);
+                const bool items_w = wp.NT && !wp.w.dbuf;   // one partial per strip and band
+                const int tiles_x = use_strip ? 1 : items_w ? wp.w.strips : (w + tx - 1) / tx;
+                const int tiles = use_strip ? 1 : items_w ? wp.w.strips * wp.w.bands : tiles_x * ((h + ty - 1) / ty);
                 int *cur = (k & 1) ? list1 : list0, *nxt = (k & 1) ? list0 : list1;
                 IterArgs a;
                 a.Ftest = tl[l];
@@ -1895,8 +2002,9 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
                 a.taps = taps;
                 a.px_count = hr_prof_pixiters(ctx);
                 a.err = ctx->d_err;
-                a.mtex = use_strip ? mtex : 0;
-                if (use_strip) e2 = launch_strip(ctx, k > 0, a, B, st);
+                a.mtex = use_strip || wp.NT ? mtex : 0;
+                if (wp.NT) e2 = launch_wide(ctx, wp, a, tile_tx, tile_ty, use_tma ? kVarNT[var] : kIterThreads, !use_tma, B, st);
+                else if (use_strip) e2 = launch_strip(ctx, k > 0, a, B, st);
                 else if (tma_k) e2 = dispatch_iter_tma(ctx, rad, var, k > 0, k > 0 ? tmS[k & 1] : tmS[2], tmF, a, B * tiles, st);
                 else e2 = dispatch_iter(ctx, rad, a, B * tiles, st);
                 if (e2) return e2;
@@ -1979,11 +2087,11 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
         // graph key: everything the launches of this level depend on
         hr_graph_key key{};
         const void *kp[] = {ref_idx, tl[l], rl[l], u0, s0, s1, uout, part, hist, lists, iters, status, field,
-                            ctx->d_err, (const void *)(uintptr_t)mtex};
+                            ctx->d_err, (const void *)(uintptr_t)mtex, wp.w.dbuf};
         static_assert(sizeof(kp) / sizeof(kp[0]) <= sizeof(key.p) / sizeof(key.p[0]), "graph key");
         for (size_t i = 0; i < sizeof(kp) / sizeof(kp[0]); ++i) key.p[i] = kp[i];
         const int ki[] = {l, L, B, h, w, cap, cap_max, rad, var, (int)use_tma, p->stop_window, (int)use_strip,
-                          (int)use_loop, (int)use_level, plan.C};
+                          (int)use_loop, (int)use_level, plan.C, wp.NT};
         for (size_t i = 0; i < sizeof(ki) / sizeof(ki[0]); ++i) key.i[i] = ki[i];
         key.f[0] = p->alpha;
         key.f[1] = p->stop_tol;

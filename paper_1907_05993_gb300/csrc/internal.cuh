@@ -83,6 +83,7 @@ struct hrebsd_ctx {
     int cnn_tc = 1;      // learned initialiser: 3x3 convolutions on tcgen05 (else mma.sync kernels)
     int tex_gather = 1;  // row sweep: moving image by texture gathers from a CUDA array copy (else plain loads)
     int tex_max_rows = 0;         // texture-gather array height limit of the device (0 = not queried)
+    int tex_max_cols = 0;         // and its width limit
     std::vector<hr_mtex> mtex;    // reference arrays per level width
     cudaStream_t cap_stream = nullptr;   // private stream the graphs are captured on
     std::vector<hr_graph_entry> graph_cache;
