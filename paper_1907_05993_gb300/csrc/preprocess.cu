@@ -1,24 +1,30 @@
 // a1: static background correction + normalisation, and the 2x2 pyramid.
 //
 // Section 2 normalises every pattern to zero mean before correlation and
-// Section 3.3 corrects the background before registration.  One CTA owns one
+// Section 3.3 corrects the background before registration.  One CTA (a cluster
+// of them where there are few patterns) owns one
 // pattern: it reads it for the background moments, divides it by the fitted
 // quadric once (float-float) writing the quotient less a constant to the
-// output, then reads that back for the variance and the normalised output;
-// the pattern (at most a few hundred KB) stays in L2 between the passes, so
-// HBM sees between one read and one write per pixel and twice that (the CTAs'
-// patterns together exceed L2).  Bound by instruction issue (188 per pixel, a
-// third of them float-float arithmetic): 4,096 patterns of 256 x 256 1.59 ms,
+// output, then reads that back for the variance and the normalised output.
+// The pattern stays in L2 between the passes as far as the patterns in work fit
+// together; what is read or written for the last time is marked to leave first
+// (HBM sees 2.2 reads and 1.5 writes a pixel, 3.3 and 1.9 without the marks).
+// 4,096 patterns of 256 x 256: 1.02 ms, bound by the latency of the passes' loads
+// (L2 and HBM, 46 % of the issue slots used, 86 instructions a pixel); 1.23 ms
+// without the marks, 1.59 ms with scalar float-float arithmetic, index
+// arithmetic for every pixel and a pass over the fit's sign (188 instructions),
 // 2.40 ms with one load in flight per thread, an integer division per pixel
 // and pass and the chunk sums in FP64.
 #include <math.h>
 #include <string.h>
 
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace {
 
-constexpr int kPreThreads = 512;
+constexpr int kPreThreads = 512, kPreChunk = 8;
 
 struct QuadricInverse {
     double ginv[36];   // inverse Gram matrix of the basis {1, x, y, x^2, xy, y^2}
@@ -107,19 +113,48 @@ __device__ __forceinline__ ff two_sum(float a, float b)
     return {s, e};
 }
 
-__device__ __forceinline__ ff ff_add(ff a, ff b)
+// The same where a is zero or a multiple of the last place of b, or |a| >= |b| (Dekker's fast two-sum):
+// three operations, the same pair.
+__device__ __forceinline__ ff fast_two_sum(float a, float b)
 {
-    ff s = two_sum(a.hi, b.hi);
-    const float lo = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
-    return two_sum(s.hi, lo);
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
 }
 
-__device__ __forceinline__ ff ff_mul(ff a, ff b)
+// Two pixels' float-float numbers at a time, in packed FP32x2 arithmetic (a - b as fma(b, -1, a)); every
+// rounding step is the scalar one.
+struct ff2 {
+    float2 hi, lo;
+};
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, both(-1.0f), a); }
+__device__ __forceinline__ ff2 two_sum(float2 a, float2 b)
 {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = __fmaf_rn(a.hi, b.hi, -p);   // exact error of the product
-    e = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, e));
-    return two_sum(p, e);
+    const float2 s = __fadd2_rn(a, b), bb = sub2(s, a);
+    return {s, __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+__device__ __forceinline__ ff2 fast_two_sum(float2 a, float2 b)
+{
+    const float2 s = __fadd2_rn(a, b);
+    return {s, sub2(b, sub2(s, a))};
+}
+
+// The last step of a sum: s.hi is a multiple of the smaller last place of a.hi and b.hi; where that is not
+// one of lo's, one of them is 2^20 times the other and |s.hi| > |lo|.
+__device__ __forceinline__ ff2 ff_add(ff2 a, ff2 b)
+{
+    const ff2 s = two_sum(a.hi, b.hi);
+    return fast_two_sum(s.hi, __fadd2_rn(s.lo, __fadd2_rn(a.lo, b.lo)));
+}
+
+// a b, na = -a.hi.  (The error term of a product is at most a few of its last places.)
+__device__ __forceinline__ ff2 ff_mul(ff2 a, float2 na, ff2 b)
+{
+    const float2 np = __fmul2_rn(na, b.hi);                // minus the product
+    float2 e = __ffma2_rn(a.hi, b.hi, np);                 // its exact error
+    e = __ffma2_rn(a.hi, b.lo, __ffma2_rn(a.lo, b.hi, e));
+    const float2 s = sub2(e, np);                          // fast_two_sum(-np, e)
+    return {s, sub2(e, __fadd2_rn(s, np))};
 }
 
 // A running sum of FP32 terms in three parts with exact carries (~72 bits): what a sum in FP64 holds,
@@ -135,7 +170,17 @@ struct Sum3 {
         s1 = b.hi;
         s2 = __fadd_rn(s2, b.lo);
     }
-    __device__ __forceinline__ double value() const { return (double)s0 + ((double)s1 + (double)s2); }
+};
+struct Sum3x2 {   // two of them
+    float2 s0 = {0.0f, 0.0f}, s1 = {0.0f, 0.0f}, s2 = {0.0f, 0.0f};
+    __device__ __forceinline__ void add(float2 v)
+    {
+        const ff2 a = two_sum(s0, v);
+        s0 = a.hi;
+        const ff2 b = two_sum(s1, a.lo);
+        s1 = b.hi;
+        s2 = __fadd2_rn(s2, b.lo);
+    }
 };
 
 // coordinate (2 k + 1 - n) / n in [-1, 1] of pixel k of n as hi + lo
@@ -149,73 +194,184 @@ __device__ __forceinline__ ff pixel_coord(int k, int n)
 
 constexpr int kMaxDim = 1536;   // largest H and W of the background fit (per-row and per-column terms in shared memory)
 
-__global__ void __launch_bounds__(kPreThreads, 3) preprocess_kernel(const float *__restrict__ in, float *out, int H,
+__device__ __forceinline__ unsigned cluster_reg(bool size)
+{
+    unsigned r;
+    if (size) asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    else asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Value at the shared-memory address `p` of this CTA in the CTA of rank `r`.
+template <class T>
+__device__ __forceinline__ T remote(const T *p, unsigned r)
+{
+    static_assert(sizeof(T) == 4 || sizeof(T) == 8, "float or double");
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("mapa.shared::cluster.u32 %0, %0, %1;" : "+r"(a) : "r"(r));
+    T v;
+    if constexpr (sizeof(T) == 4) asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    else asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+    return v;
+}
+
+// COL: the width divides the CTA's threads, so that a thread's pixels lie in one column.
+// CL: a cluster of CTAs shares the pattern, the chunks dealt out in turn.  The threads' partial sums of the
+// ranks are added exactly (Sum3), thread by thread, in rank 0, so that they are the sums of one CTA.
+template <bool COL, bool CL>
+__global__ void __launch_bounds__(kPreThreads, CL ? 2 : 3) preprocess_kernel(const float *__restrict__ in, float *out, int H,
                                                                  int W, int flat, QuadricInverse qi)
 {
+    extern __shared__ float sums[];   // CL: the threads' partial sums [18][kPreThreads]
+    const unsigned csize = CL ? cluster_reg(true) : 1, rank = CL ? cluster_reg(false) : 0;
     __shared__ double red[32 * 6];
-    __shared__ double coef[6];
+    __shared__ double coef[7];   // the quadric's coefficients, the pattern's sum
     __shared__ float2 rowA[kMaxDim], rowB[kMaxDim];   // per row: c0 + c2 y + c5 y^2 and c1 + c4 y (hi, lo)
-    __shared__ float2 colX[kMaxDim];                  // per column: x (hi, lo)
+    __shared__ float2 colX[COL ? 1 : kMaxDim];        // per column: x (hi, lo)
     __shared__ float rowY[kMaxDim];                   // per row: y (the correctly rounded FP32 coordinate)
-    const size_t base = (size_t)blockIdx.x * H * W;
+    const size_t base = (size_t)(CL ? blockIdx.x / csize : blockIdx.x) * H * W;
     const float *img = in + base;
+    constexpr int bd = kPreThreads;
+    const int t = threadIdx.x;
     auto row_of = [&](int p) { return (int)__umulhi((unsigned)p, qi.mw); };
-    const int n = H * W;
+    const int n = H * W, rstep = COL ? bd / W : 0;   // COL: rows between a thread's pixels
 
     // Sums are taken in FP32 over chunks of kChunk pixels of one thread, the chunk sums added exactly and
     // the threads' sums in FP64: the quadric's coefficients come out of a poorly conditioned 6 x 6 system, and plain FP32
     // sums of ~128 terms would move the output by ~1e-4.
-    constexpr int kChunk = 8;
+    constexpr int kChunk = kPreChunk;
+    ff xt{0.0f, 0.0f};   // COL: the thread's column
     if (flat) {   // the pixel coordinates, once per row and column
-        for (int j = threadIdx.x; j < W; j += blockDim.x) {
-            const ff x = pixel_coord(j, W);
-            colX[j] = make_float2(x.hi, x.lo);
-        }
-        for (int i = threadIdx.x; i < H; i += blockDim.x) rowY[i] = pixel_coord(i, H).hi;
+        if (COL) xt = pixel_coord(t % W, W);
+        else
+            for (int j = t; j < W; j += bd) {
+                const ff x = pixel_coord(j, W);
+                colX[j] = make_float2(x.hi, x.lo);
+            }
+        for (int i = t; i < H; i += bd) rowY[i] = pixel_coord(i, H).hi;
         __syncthreads();
     }
-    // A chunk's pixels are loaded before any of them is used (past the end: the last pixel, counted as 0),
-    // so that a thread has kChunk loads in flight: the passes are bound by memory latency otherwise.
-    const int bd = blockDim.x;
-    auto load = [&](const float *src, int p0, float (&v)[kChunk]) {
+    // f(p0, whole) for the chunks p0, p0 + bd, ... of this thread; whole: every pixel is inside (else f counts
+    // the others as 0).  A chunk's pixels are loaded before any of them is used, so that a thread has kChunk
+    // loads in flight: the passes are bound by memory latency otherwise.
+    auto chunks = [&](auto f) {
+        int p0 = t + (int)rank * (kChunk * bd);
+        for (; p0 + (kChunk - 1) * bd < n; p0 += (int)csize * (kChunk * bd)) f(p0, std::true_type());
+        if (p0 < n) f(p0, std::false_type());
+    };
+    // last: read for the last time (the line is the first to leave L2)
+    auto load = [&](const float *src, int p0, auto whole, float (&v)[kChunk], auto last) {
 #pragma unroll
-        for (int c = 0; c < kChunk; ++c) v[c] = src[min(p0 + c * bd, n - 1)];
+        for (int c = 0; c < kChunk; ++c)
+            v[c] = whole || p0 + c * bd < n ? (last ? __ldcs(src + p0 + c * bd) : src[p0 + c * bd]) : 0.0f;
+    };
+    // row and column of a chunk's pixel c (past the end: the last row); i0 = row_of(p0)
+    auto cell = [&](int p0, int i0, int c, auto whole, int &i, int &j) {
+        if (COL) {
+            i = i0 + c * rstep;
+            if (!whole) i = min(i, H - 1);
+            j = 0;
+        } else {
+            const int p = whole ? p0 + c * bd : min(p0 + c * bd, n - 1);
+            i = c == 0 ? i0 : row_of(p);
+            j = p - i * W;
+        }
+    };
+    // CL: thread t's parts x[0 .. NF) (three per sum) of all ranks added in rank 0; the caller meets once more
+    // before `sums` is written again
+    auto merge = [&](auto *x, auto nf) {
+        constexpr int NF = decltype(nf)::value;
+        if (!CL) return;
+#pragma unroll
+        for (int k = 0; k < NF; ++k) sums[k * bd + t] = x[k];
+        cluster_sync();
+        if (rank == 0)
+            for (unsigned r = 1; r < csize; ++r) {
+                float y[NF];
+#pragma unroll
+                for (int k = 0; k < NF; ++k) y[k] = remote(sums + k * bd + t, r);
+#pragma unroll
+                for (int k = 0; k < NF; k += 3) {
+                    Sum3 s{x[k], x[k + 1], x[k + 2]};
+                    s.add(y[k]);
+                    s.add(y[k + 1]);
+                    s.add(y[k + 2]);
+                    x[k] = s.s0;
+                    x[k + 1] = s.s1;
+                    x[k + 2] = s.s2;
+                }
+            }
+    };
+    auto value3 = [](const float *x) { return (double)x[0] + ((double)x[1] + (double)x[2]); };
+    // one sum over the pattern, in every thread of the cluster
+    auto total_of = [&](const Sum3 &part) {
+        float x[3] = {part.s0, part.s1, part.s2};
+        merge(x, std::integral_constant<int, 3>());
+        double s[1] = {value3(x)};
+        block_sum<1>(s, red);
+        if (CL) {
+            if (t == 0) coef[0] = s[0];
+            cluster_sync();
+            if (rank) s[0] = remote(coef, 0);
+            cluster_sync();
+        }
+        return s[0];
     };
     // pass 1: quadric moments b_k = sum phi_k I (basis at the correctly rounded pixel coordinates);
     // b_0 is the pattern's sum
     double total = 0.0;
     if (flat) {
-        Sum3 part[6];
-        for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * blockDim.x) {
+        Sum3x2 part[3];
+        chunks([&](int p0, auto whole) {
             float acc[6] = {0, 0, 0, 0, 0, 0}, v[kChunk];
-            load(img, p0, v);
+            load(img, p0, whole, v, std::false_type());
+            const int i0 = row_of(p0);
 #pragma unroll
             for (int c = 0; c < kChunk; ++c) {
-                const int p = min(p0 + c * bd, n - 1), i = row_of(p), j = p - i * W;
-                const float vc = p0 + c * bd < n ? v[c] : 0.0f;
+                int i, j;
+                cell(p0, i0, c, whole, i, j);
                 float phi[6];
-                basis6(colX[j].x, rowY[i], phi);
+                basis6(COL ? xt.hi : colX[j].x, rowY[i], phi);
 #pragma unroll
-                for (int k = 0; k < 6; ++k) acc[k] = fmaf(phi[k], vc, acc[k]);
+                for (int k = 0; k < 6; ++k) acc[k] = fmaf(phi[k], v[c], acc[k]);
             }
 #pragma unroll
-            for (int k = 0; k < 6; ++k) part[k].add(acc[k]);
+            for (int k = 0; k < 3; ++k) part[k].add(make_float2(acc[2 * k], acc[2 * k + 1]));
+        });
+        float x[18];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            x[3 * k] = k % 2 ? part[k / 2].s0.y : part[k / 2].s0.x;
+            x[3 * k + 1] = k % 2 ? part[k / 2].s1.y : part[k / 2].s1.x;
+            x[3 * k + 2] = k % 2 ? part[k / 2].s2.y : part[k / 2].s2.x;
         }
+        merge(x, std::integral_constant<int, 18>());
         double d[6];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) d[k] = part[k].value();
+        for (int k = 0; k < 6; ++k) d[k] = value3(x + 3 * k);
         block_sum<6>(d, red);
-        total = d[0];
-        if (threadIdx.x == 0) {
+        if (t == 0) {
             for (int r = 0; r < 6; ++r) {
                 double c = 0.0;
                 for (int k = 0; k < 6; ++k) c += qi.ginv[r * 6 + k] * d[k];
                 coef[r] = c;
             }
+            coef[6] = d[0];
+        }
+        if (CL) {   // rank 0's coefficients and sum in every CTA
+            cluster_sync();
+            double c = 0.0;
+            if (rank && t < 7) c = remote(coef + t, 0);
+            cluster_sync();
+            if (rank && t < 7) coef[t] = c;
         }
         __syncthreads();
+        total = coef[6];
         // per-row parts of the quadric in FP64, kept as hi + lo
-        for (int i = threadIdx.x; i < H; i += blockDim.x) {
+        for (int i = t; i < H; i += bd) {
             const double y = (2.0 * i + 1.0 - H) / H;
             const ff A = ff_from_double(coef[0] + y * (coef[2] + y * coef[5]));
             const ff Bc = ff_from_double(coef[1] + y * coef[4]);
@@ -226,102 +382,126 @@ __global__ void __launch_bounds__(kPreThreads, 3) preprocess_kernel(const float 
     }
     const ff C = flat ? ff_from_double(coef[3]) : ff{0.0f, 0.0f};
 
-    // the quadric at pixel p as hi + lo: A(y) + x (B(y) + x c3)
-    auto fit_at = [&](int p) -> ff {
-        const int i = row_of(p), j = p - i * W;
-        const ff x = {colX[j].x, colX[j].y};
-        const ff A = {rowA[i].x, rowA[i].y}, Bc = {rowB[i].x, rowB[i].y};
-        return ff_add(A, ff_mul(x, ff_add(Bc, ff_mul(x, C))));
-    };
     // the division is skipped when the fitted surface is not positive at every pixel (checked on the
-    // FP32 value of the quadric, whose sign differs from the hi + lo one only within rounding of zero)
+    // FP32 value of the quadric, whose sign differs from the hi + lo one only within rounding of zero);
+    // no pixel needs a look where every row's lower bound is clear of the rounding (3 x 2^-24 of its terms)
     bool use_fit = flat;
     if (flat) {
         bool bad = false;
-#pragma unroll 4
-        for (int p = threadIdx.x; p < n; p += blockDim.x) {
-            const int i = row_of(p), j = p - i * W;
-            const float x = colX[j].x;
-            bad |= !(fmaf(x, fmaf(x, C.hi, rowB[i].x), rowA[i].x) > 0.0f);
+        for (int i = t; i < H; i += bd) {
+            const float a = rowA[i].x, b = fabsf(rowB[i].x), low = a - b - fmaxf(-C.hi, 0.0f);
+            bad |= !(low > 1e-5f * (a + b + fabsf(C.hi)));
         }
-        use_fit = !__syncthreads_or(bad);
+        if (__syncthreads_or(bad)) {
+            bad = false;
+#pragma unroll 4
+            for (int p = t; p < n; p += bd) {
+                const int i = row_of(p);
+                const float x = COL ? xt.hi : colX[p - i * W].x;
+                bad |= !(fmaf(x, fmaf(x, C.hi, rowB[i].x), rowA[i].x) > 0.0f);
+            }
+            use_fit = !__syncthreads_or(bad);
+        }
     }
 
-    // the pattern divided by the quadric, as hi + lo: q ~ v / f (within 2 units of the last place,
-    // from the correctly rounded reciprocal), the remainder v - q f.hi exact by fma, then the
+    // pass 2: the pattern divided by the quadric A(y) + x (B(y) + x c3), as hi + lo: q ~ v / f (within 2 units
+    // of the last place, from the correctly rounded reciprocal), the remainder v - q f.hi exact by fma, then the
     // correction (remainder - q f.lo) / f; with the division by f.hi a product with the same
-    // reciprocal (its error lands ~2^-24 below the correction, itself ~2^-24 below q)
-    auto value = [&](int p, float v) -> ff {
-        if (!use_fit) return {v, 0.0f};
-        const ff f = fit_at(p);
-        const float rf = __frcp_rn(f.hi);
-        const float q = __fmul_rn(v, rf);
-        float r = __fmaf_rn(-q, f.hi, v);
-        r = __fmaf_rn(-q, f.lo, r);
-        return two_sum(q, __fmul_rn(r, rf));
-    };
-    // pass 2: the quotient less K (1 for the background-divided pattern, whose values lie near one;
+    // reciprocal (its error lands ~2^-24 below the correction, itself ~2^-24 below q).  Of it the quotient
+    // less K (1 for the background-divided pattern, whose values lie near one;
     // the mean intensity, rounded, for the raw one), d = (q.hi - K) + q.lo in FP32: the leading part
     // cancels before rounding, so d keeps the float-float accuracy of q and the mean of d is small; d
     // is stored in the output (the pattern is read before it is overwritten, by the same thread) and
     // summed for the mean
     if (!flat) {   // the raw pattern's sum for K
         Sum3 part;
-        for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * blockDim.x) {
+        chunks([&](int p0, auto whole) {
             float sv = 0.0f, v[kChunk];
-            load(img, p0, v);
+            load(img, p0, whole, v, std::false_type());
 #pragma unroll
-            for (int c = 0; c < kChunk; ++c) sv += p0 + c * bd < n ? v[c] : 0.0f;
+            for (int c = 0; c < kChunk; ++c) sv += v[c];
             part.add(sv);
-        }
-        double t[1] = {part.value()};
-        block_sum<1>(t, red);
-        total = t[0];
+        });
+        total = total_of(part);
     }
     const float K = use_fit ? 1.0f : (float)(total / n);
     float *o = out + base;
     Sum3 sum_d;
-    for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * blockDim.x) {
-        float sd = 0.0f, v[kChunk];
-        load(img, p0, v);
+    if (use_fit) {
+        const ff2 C2 = {both(C.hi), both(C.lo)};
+        const ff2 x1 = {both(xt.hi), both(xt.lo)}, xC1 = ff_mul(x1, both(-xt.hi), C2);
+        chunks([&](int p0, auto whole) {
+            float sd = 0.0f, v[kChunk];
+            load(img, p0, whole, v, std::true_type());
+            const int i0 = row_of(p0);
 #pragma unroll
-        for (int c = 0; c < kChunk; ++c) {
-            const int p = min(p0 + c * bd, n - 1);
-            const ff q = value(p, v[c]);
-            const float d = __fadd_rn(__fsub_rn(q.hi, K), q.lo);
-            if (p0 + c * bd < n) o[p] = d;
-            sd += p0 + c * bd < n ? d : 0.0f;
-        }
-        sum_d.add(sd);
+            for (int c = 0; c < kChunk; c += 2) {   // two pixels at a time
+                int i, j, i2, j2;
+                cell(p0, i0, c, whole, i, j);
+                cell(p0, i0, c + 1, whole, i2, j2);
+                const float2 a = rowA[i], a2 = rowA[i2], b = rowB[i], b2 = rowB[i2];
+                ff2 x = x1, xC = xC1;
+                float2 nx = both(-xt.hi);
+                if (!COL) {
+                    const float2 xa = colX[j], xb = colX[j2];
+                    x = {make_float2(xa.x, xb.x), make_float2(xa.y, xb.y)};
+                    nx = __fmul2_rn(x.hi, both(-1.0f));
+                    xC = ff_mul(x, nx, C2);
+                }
+                const ff2 A = {make_float2(a.x, a2.x), make_float2(a.y, a2.y)}, Bc = {make_float2(b.x, b2.x), make_float2(b.y, b2.y)};
+                const ff2 f = ff_add(A, ff_mul(x, nx, ff_add(Bc, xC)));
+                const float2 vv = make_float2(v[c], v[c + 1]);
+                const float2 rf = make_float2(__frcp_rn(f.hi.x), __frcp_rn(f.hi.y));
+                const float2 q = __fmul2_rn(vv, rf), nq = __fmul2_rn(q, both(-1.0f));
+                const float2 r = __ffma2_rn(nq, f.lo, __ffma2_rn(nq, f.hi, vv));
+                const ff2 e = fast_two_sum(q, __fmul2_rn(r, rf));
+                const float2 d = __fadd2_rn(__fadd2_rn(e.hi, both(-K)), e.lo);
+                if (whole || p0 + c * bd < n) o[p0 + c * bd] = d.x;
+                if (whole || p0 + (c + 1) * bd < n) o[p0 + (c + 1) * bd] = d.y;
+                sd += whole || p0 + c * bd < n ? d.x : 0.0f;
+                sd += whole || p0 + (c + 1) * bd < n ? d.y : 0.0f;
+            }
+            sum_d.add(sd);
+        });
+    } else {
+        chunks([&](int p0, auto whole) {
+            float sd = 0.0f, v[kChunk];
+            load(img, p0, whole, v, std::true_type());
+#pragma unroll
+            for (int c = 0; c < kChunk; ++c) {
+                const float d = __fadd_rn(__fsub_rn(v[c], K), 0.0f);
+                if (whole || p0 + c * bd < n) {
+                    o[p0 + c * bd] = d;
+                    sd += d;
+                }
+            }
+            sum_d.add(sd);
+        });
     }
-    double m[1] = {sum_d.value()};
-    block_sum<1>(m, red);
-    const double mean_d = m[0] / n, mean = mean_d + (double)K;
+    const double mean_d = total_of(sum_d) / n, mean = mean_d + (double)K;
     const float md = (float)mean_d;
     // pass 3: variance about the mean
     Sum3 sum_v;
-    for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * blockDim.x) {
+    chunks([&](int p0, auto whole) {
         float ss = 0.0f, v[kChunk];
-        load(o, p0, v);
+        load(o, p0, whole, v, std::false_type());
 #pragma unroll
         for (int c = 0; c < kChunk; ++c) {
-            const float d = p0 + c * bd < n ? __fsub_rn(v[c], md) : 0.0f;
+            const float d = whole || p0 + c * bd < n ? __fsub_rn(v[c], md) : 0.0f;
             ss = fmaf(d, d, ss);
         }
         sum_v.add(ss);
-    }
-    double v2[1] = {sum_v.value()};
-    block_sum<1>(v2, red);
-    const double sdv = sqrt(v2[0] / n);
+    });
+    const double sdv = sqrt(total_of(sum_v) / n);
     const float inv = (sdv > 0.0 && sdv > 1e-6 * fabs(mean)) ? (float)(1.0 / sdv) : 0.0f;
     // pass 4: output
-    for (int p0 = threadIdx.x; p0 < n; p0 += kChunk * bd) {
+    chunks([&](int p0, auto whole) {
         float v[kChunk];
-        load(o, p0, v);
+        load(o, p0, whole, v, std::true_type());
 #pragma unroll
         for (int c = 0; c < kChunk; ++c)
-            if (p0 + c * bd < n) o[p0 + c * bd] = __fsub_rn(v[c], md) * inv;
-    }
+            if (whole || p0 + c * bd < n) __stcs(o + p0 + c * bd, __fsub_rn(v[c], md) * inv);
+    });
 }
 
 // One pyramid level down: the 2x2 box mean, floor(H/2) x floor(W/2) (an odd
@@ -440,7 +620,31 @@ extern "C" int hrebsd_preprocess_batch(hrebsd_ctx *ctx, const float *in, int n, 
     if (!flat)
         for (double &g : qi.ginv) g = 0.0;
     hr_prof_begin(ctx, hr_stream(stream));
-    preprocess_kernel<<<n, kPreThreads, 0, hr_stream(stream)>>>(in, out, H, W, flat, qi);
+    // few patterns: a cluster of up to 8 CTAs on each, while two CTAs per SM hold them all and each has at least
+    // four chunks.  One CTA -> cluster: one 1244 x 1024 908 -> 137 us, 60 of them 1,556 -> 492 us, 10 of 640 x 480
+    // 239 -> 62 us, one 256 x 256 63 -> 38 us.  Beyond the rule: 200 of 256 x 256, which keep the SMs busy without,
+    // 103 -> 98 us in pairs and 147 us in fours; one 128 x 128, of four chunks, 30 -> 32 us
+    int C = 8;
+    while (C > 1 && ((long long)n * C > 2 * ctx->num_sms || (long long)H * W < 4LL * C * kPreChunk * kPreThreads)) C /= 2;
+    // widths that divide the CTA (64, 128, 256 ...): the column's terms once per thread
+    const bool col = kPreThreads % W == 0;
+    auto k = C > 1 ? (col ? preprocess_kernel<true, true> : preprocess_kernel<false, true>)
+                   : (col ? preprocess_kernel<true, false> : preprocess_kernel<false, false>);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(n * C));
+    cfg.blockDim = dim3(kPreThreads);
+    cfg.stream = hr_stream(stream);
+    cudaLaunchAttribute at;
+    if (C > 1) {
+        cfg.dynamicSmemBytes = 18 * kPreThreads * sizeof(float);
+        HR_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)C;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+    }
+    HR_CHECK(cudaLaunchKernelEx(&cfg, k, in, out, H, W, flat, qi));
     hr_prof_end(ctx, PROF_PRE, hr_stream(stream));
     HR_LAUNCHED(ctx);
     return HREBSD_OK;
