@@ -281,7 +281,9 @@ __global__ void __launch_bounds__(NT, 1) demons_cluster_kernel(const __grid_cons
             F[p] = Fg[(size_t)clampi(lo + y - 1, 0, h - 1) * w + x];
         }
         if (t == 0) s_state = CONTINUE;
-        __syncthreads();
+        // the whole cluster, not only this CTA: iteration 0 stores into the neighbours' shared memory without
+        // a barrier in between, which is defined only once every CTA of the cluster runs
+        sync_all();
         for (int k = 0;; ++k) {
             bool final_pass = false;
             if (k > 0) {
