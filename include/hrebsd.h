@@ -317,7 +317,9 @@ int hrebsd_remap(hrebsd_ctx *ctx, const float *ref, const int32_t *ref_idx, cons
  * (0.5 (1 - cos(2 pi n/(S-1)))), c = IFFT(FFT(test) conj(FFT(ref))), i.e.
  * c(s) = sum_x test(x+s) ref(x); integer peak = first maximum in row-major
  * order, wrapped to [-S/2, S/2); sub-pixel 3-point parabola per axis.
- * S in {16, 32, 64, 128}; ROIs must lie inside the image.  Outputs
+ * S in {16, 32, 64, 128, 256}.  A ROI that reaches outside the image, or that
+ * holds a non-finite pixel (its whole correlation is then NaN), gets q = NaN,
+ * peak = 0, peak_height = 0, near_tie = 0.  Outputs
  * q [B][N][2] (x, y shift: test(x + q) ~ ref(x)), peak [B][N][2],
  * peak_height [B][N] (c0 / (|ref_w| |test_w|)), near_tie [B][N] (top two
  * correlation values within 1e-6 |c0|; may be NULL). */

@@ -79,6 +79,16 @@ __device__ float block_sum(float v, float *red)
 // (value, index) ordering: larger value first, then smaller index.
 __device__ __forceinline__ bool better(float v, int i, float bv, int bi) { return v > bv || (v == bv && i < bi); }
 
+// A ROI without a peak: one that reaches outside the image, or one whose correlation holds no comparable value
+// (a single NaN pixel makes all of it NaN, through the mean; `better` then leaves the start index 0x7fffffff).
+__device__ __forceinline__ void write_no_peak(size_t o, float *q, int32_t *peak, float *ph, int32_t *near_tie)
+{
+    q[2 * o] = q[2 * o + 1] = __int_as_float(0x7fc00000);
+    peak[2 * o] = peak[2 * o + 1] = 0;
+    ph[o] = 0.0f;
+    if (near_tie) near_tie[o] = 0;
+}
+
 template <int S, int NT>
 __global__ void __launch_bounds__(NT) xcf_kernel(const float *__restrict__ rem, const float *__restrict__ test, int B,
                                                  int H, int W, const int32_t *__restrict__ roi, int N, int window,
@@ -96,12 +106,7 @@ __global__ void __launch_bounds__(NT) xcf_kernel(const float *__restrict__ rem, 
     const int x0 = cx - S / 2, y0 = cy - S / 2;
     const size_t o = (size_t)blockIdx.x;
     if (x0 < 0 || y0 < 0 || x0 + S > W || y0 + S > H) {   // ROI outside the image
-        if (threadIdx.x == 0) {
-            q[2 * o] = q[2 * o + 1] = __int_as_float(0x7fc00000);
-            peak[2 * o] = peak[2 * o + 1] = 0;
-            ph[o] = 0.0f;
-            if (near_tie) near_tie[o] = 0;
-        }
+        if (threadIdx.x == 0) write_no_peak(o, q, peak, ph, near_tie);
         return;
     }
     for (int j = threadIdx.x; j < S / 2; j += NT) {
@@ -198,6 +203,10 @@ __global__ void __launch_bounds__(NT) xcf_kernel(const float *__restrict__ rem, 
             } else {
                 v2 = fmaxf(v2, rv[k]);
             }
+        }
+        if (i >= S * S) {   // every value is a NaN
+            write_no_peak(o, q, peak, ph, near_tie);
+            return;
         }
         const int py = i / S, px = i % S;
         const float c0 = v;
@@ -332,12 +341,7 @@ __global__ void __launch_bounds__(NT, 2) xcf64_kernel(const float *__restrict__ 
     const int x0 = cx - S / 2, y0 = cy - S / 2;
     const size_t o = (size_t)blockIdx.x;
     if (x0 < 0 || y0 < 0 || x0 + S > W || y0 + S > H) {   // ROI outside the image
-        if (threadIdx.x == 0) {
-            q[2 * o] = q[2 * o + 1] = __int_as_float(0x7fc00000);
-            peak[2 * o] = peak[2 * o + 1] = 0;
-            ph[o] = 0.0f;
-            if (near_tie) near_tie[o] = 0;
-        }
+        if (threadIdx.x == 0) write_no_peak(o, q, peak, ph, near_tie);
         return;
     }
     if (threadIdx.x < S) {
@@ -459,6 +463,10 @@ __global__ void __launch_bounds__(NT, 2) xcf64_kernel(const float *__restrict__ 
             } else {
                 v2 = fmaxf(v2, rv[k]);
             }
+        }
+        if (i >= S * S) {   // every value is a NaN
+            write_no_peak(o, q, peak, ph, near_tie);
+            return;
         }
         const int py = i / S, px = i % S;
         const float c0 = v;
@@ -747,12 +755,7 @@ __global__ void __launch_bounds__(NT, 3) peak_kernel(const float2 *__restrict__ 
     const size_t o = (size_t)b0 * N + lr;
     const float nt = norms[2 * lr], nr = norms[2 * lr + 1];
     if (nt < 0.0f) {
-        if (threadIdx.x == 0) {
-            q[2 * o] = q[2 * o + 1] = __int_as_float(0x7fc00000);
-            peak[2 * o] = peak[2 * o + 1] = 0;
-            ph[o] = 0.0f;
-            if (near_tie) near_tie[o] = 0;
-        }
+        if (threadIdx.x == 0) write_no_peak(o, q, peak, ph, near_tie);
         return;
     }
     twiddles(tw);
@@ -820,6 +823,10 @@ __global__ void __launch_bounds__(NT, 3) peak_kernel(const float2 *__restrict__ 
     __syncthreads();
     // the correlation's rows around the peak once more
     const int i = s_i, py = i / S, px = i % S;
+    if (i >= S * S) {   // every value is a NaN
+        if (threadIdx.x == 0) write_no_peak(o, q, peak, ph, near_tie);
+        return;
+    }
     for (int k = 0; k < 3; ++k) zs[k * LS + at(threadIdx.x)] = Zr[(size_t)((py + S - 1 + k) & (S - 1)) * S + threadIdx.x];
     __syncthreads();
     fft_lines(zs, 3, tw, +1);
