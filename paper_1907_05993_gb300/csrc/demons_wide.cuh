@@ -4,9 +4,9 @@
 //
 // An item is a strip of at most NT - 15 output columns and a band of rows of one active pair.  Thread t owns
 // the image column xl + t of the strip's loaded columns; u is exact from 3 columns inside, du's x pass from 6.
-// Columns outside the image stand for the edge column: their threads read the edge column's x-pass rows, so
-// that they form the same u and du (the last strip's origin is shifted so that the three columns past the
-// edge lie in the edge column's warp).  A band starts 6 rows early (rows that are only pushed through the
+// The three columns past an image edge stand for the edge column: their threads read its x-pass rows, so that
+// they form the same u and du (the last strip's origin is shifted so that they lie in the edge column's
+// warp; see demons_wide_columns.cuh).  A band starts 6 rows early (rows that are only pushed through the
 // windows) unless it starts at the top, where the first row fills the windows.  The rows of a step are copied
 // by cp.async, each thread its own column (8 and 4 bytes: no alignment needed), completion on an mbarrier.
 //
@@ -25,6 +25,8 @@
 namespace wide {
 
 constexpr int R = 7, RAD = 3;
+
+#include "demons_wide_columns.cuh"
 
 template <int NT>
 struct Geo {
@@ -111,12 +113,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_wide_kernel(IterArgs a, W
         m.pair = a.active[slot];
         m.x0 = s * wa.sw;
         m.x1 = min(w, m.x0 + wa.sw);
-        m.xl = m.x0 - 2 * RAD;
-        if (m.x1 == w) {   // the three columns past the edge in the edge column's warp
-            const int past = ((w - 1 - m.xl) & 31) - 28;
-            // (a shift by d moves the edge column to a later lane; from lane 29 .. 31 it reaches lane 0 .. 2)
-            if (past > 0) m.xl -= 4 - past;
-        }
+        m.xl = strip_origin(m.x0, m.x1, w);
         m.yb = b * wa.bh;
         m.ye = min(h, m.yb + wa.bh);
         m.ys = m.yb > 0 ? m.yb - 2 * RAD : 0;
@@ -174,7 +171,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) demons_wide_kernel(IterArgs a, W
         const float2 *u0 = a.in + (size_t)m.pair * plane;
         float2 *dst = a.out + (size_t)m.pair * plane;
         const int x = m.xl + t, xq = clampi(x, 0, w - 1);
-        const int tc = min(xq - m.xl, NT - 1);   // this thread's column of the rows
+        const int tc = edge_column(m.xl, t, w);   // this thread's column of the rows
         const int tl = clampi(clampi(xq - 1, 0, w - 1) - m.xl, 0, NT - 1), tr = clampi(clampi(xq + 1, 0, w - 1) - m.xl, 0, NT - 1);
         const float tf_ = (float)xq, sx = (xq == 0 || xq == w - 1) ? 1.0f : 0.5f;
         const bool col = x >= m.x0 && x < m.x1;   // an output column
