@@ -1783,7 +1783,7 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
     int cap_max = 0;
     for (int l = 0; l < L; ++l) cap_max = p->max_iters[l] > cap_max ? p->max_iters[l] : cap_max;
     const int rad = max(hr_gauss_radius(p->sigma_update), hr_gauss_radius(p->sigma_field));
-    Taps taps;
+    Taps taps{};   // (zero beyond the radius: part of the graph key)
     if (hr_gauss_taps(p->sigma_update, rad, taps.up) < 0 || hr_gauss_taps(p->sigma_field, rad, taps.f) < 0)
         return HREBSD_EINVAL;
 
@@ -2084,14 +2084,18 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
             if ((e = emit(st))) return e;
             continue;
         }
-        // graph key: everything the launches of this level depend on
+        // graph key: everything the launches of this level depend on (the last of them, the prolongation, on the
+        // finer level's size: 100 and 101 rows are both 50 at the coarser one)
+        const int hf = l > 0 ? H >> (l - 1) : 0, wf = l > 0 ? W >> (l - 1) : 0;
         hr_graph_key key{};
         const void *kp[] = {ref_idx, tl[l], rl[l], u0, s0, s1, uout, part, hist, lists, iters, status, field,
                             ctx->d_err, (const void *)(uintptr_t)mtex, wp.w.dbuf};
         static_assert(sizeof(kp) / sizeof(kp[0]) <= sizeof(key.p) / sizeof(key.p[0]), "graph key");
         for (size_t i = 0; i < sizeof(kp) / sizeof(kp[0]); ++i) key.p[i] = kp[i];
         const int ki[] = {l, L, B, h, w, cap, cap_max, rad, var, (int)use_tma, p->stop_window, (int)use_strip,
-                          (int)use_loop, (int)use_level, plan.C, wp.NT};
+                          (int)use_loop, (int)use_level, plan.C, wp.NT, hf, wf};
+        static_assert(sizeof(ki) / sizeof(ki[0]) <= sizeof(key.i) / sizeof(key.i[0]), "graph key");
+        static_assert(2 + 2 * (2 * kMaxRad + 1) <= sizeof(key.f) / sizeof(key.f[0]), "graph key");
         for (size_t i = 0; i < sizeof(ki) / sizeof(ki[0]); ++i) key.i[i] = ki[i];
         key.f[0] = p->alpha;
         key.f[1] = p->stop_tol;

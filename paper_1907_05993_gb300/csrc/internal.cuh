@@ -43,7 +43,7 @@ struct hr_pending {
 // Cached CUDA graph of one pyramid level of a registration (demons.cu).
 struct hr_graph_key {
     const void *p[16];
-    int i[16];
+    int i[20];
     float f[32];
 };
 struct hr_graph_entry {
