@@ -44,6 +44,14 @@ int hr_ws(hrebsd_ctx *ctx, int slot, size_t bytes, void **out)
     return HREBSD_OK;
 }
 
+bool hr_capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 int hr_gauss_radius(float sigma)
 {
     if (!(sigma > 0.0f)) return 0;

@@ -1497,11 +1497,7 @@ int strip_capacity(hrebsd_ctx *ctx, int w)
 bool hr_graph_usable(hrebsd_ctx *ctx, cudaStream_t st)
 {
     if (!ctx->graphs || ctx->prof_on) return false;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return false;   // the caller is capturing: launch into its graph
-    }
+    if (hr_capturing(st)) return false;   // launch into the caller's graph
     if (!ctx->cap_stream && cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         ctx->cap_stream = nullptr;
@@ -1564,12 +1560,7 @@ constexpr size_t kMaxTextures = 12;   // level widths with an array
 int hr_ref_texture(hrebsd_ctx *ctx, const float *ref, int R, int h, int w, cudaStream_t st, unsigned long long *tex)
 {
     *tex = 0;
-    if (!ctx->tex_gather) return HREBSD_OK;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return HREBSD_OK;
-    }
+    if (!ctx->tex_gather || hr_capturing(st)) return HREBSD_OK;
     if (!ctx->tex_max_rows) {
         int mh = 0, mw = 0;
         HR_CHECK(cudaDeviceGetAttribute(&mh, cudaDevAttrMaxTexture2DGatherHeight, ctx->device));
@@ -1896,9 +1887,13 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
             }
             if (plan.C) wp.NT = 0;
             if (wp.NT && regroup) {
+                // no room for d, or no leave to make some (the call's other slots may be large enough already
+                // where this one is not: it is used at some batches and with a stop rule only): the tiles
+                // do without
+                const size_t bytes = (size_t)B * H * W * 4;
                 void *d = nullptr;
-                e = hr_ws(ctx, WS_DBUF, (size_t)B * H * W * 4, &d);
-                if (e == HREBSD_ENOMEM) wp.NT = 0;   // no room for d: the tiles do without
+                e = ctx->ws[WS_DBUF].bytes < bytes && hr_capturing(st) ? HREBSD_ENOMEM : hr_ws(ctx, WS_DBUF, bytes, &d);
+                if (e == HREBSD_ENOMEM) wp.NT = 0;
                 else if (e) return e;
                 wp.w.dbuf = (float *)d;
             }

@@ -114,6 +114,8 @@ static inline unsigned long long *hr_prof_pixiters(hrebsd_ctx *ctx)
 // through *out.  Allocation is synchronous (cudaMalloc) and happens only on
 // growth.
 int hr_ws(hrebsd_ctx *ctx, int slot, size_t bytes, void **out);
+// True while `st` is being captured: nothing may be allocated or synchronised then.
+bool hr_capturing(cudaStream_t st);
 int hr_set_device(hrebsd_ctx *ctx);
 
 static inline cudaStream_t hr_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
