@@ -56,6 +56,9 @@ __device__ __forceinline__ float guarded_div(float a, float d) { return fabsf(d)
 // whole blur (src, by bg too if given) by the blurred value, or subtracts that from src.
 enum { POST_NONE = 0, POST_DIV, POST_SUB };
 constexpr int RUN = 16, LINES = 32, PAIRS = LINES / 2, MAX_SEG = 256;
+// Shared memory of the largest tile.  The limit set on a kernel holds for the whole device, other handles and
+// threads included, so it is this constant and not the call's own need.
+constexpr int MAX_SMEM = PAIRS * ((MAX_SEG + 2 * kMaxFilterRadius) | 1) * (int)sizeof(float2);
 
 struct BlurArgs {
     const float *in;    // input of this pass
@@ -312,7 +315,7 @@ int launch_pass(hrebsd_ctx *ctx, const float *in, const float *src, const float 
     a.vec = (W % 2 == 0) && (reinterpret_cast<uintptr_t>(out) % 8 == 0);
     const size_t smem = (size_t)PAIRS * a.stride * sizeof(float2);
     auto k = blur_pass_kernel<AXIS, PRE, POST>;
-    if (smem > 48 * 1024) HR_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) HR_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM));
     const int threads = (runs * PAIRS + 31) / 32 * 32;   // whole warps
     const long long tiles = (a.lines + LINES - 1) / LINES * a.segs;
     for (int i0 = 0; i0 < (AXIS ? n : 1); i0 += 65535) {   // y: one image per grid row
