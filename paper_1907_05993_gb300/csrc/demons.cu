@@ -1556,7 +1556,12 @@ int hr_graph_run(hrebsd_ctx *ctx, const hr_graph_key &key, cudaStream_t st, Emit
 // height, a stream that is being captured (no allocation or synchronisation inside a capture), or an
 // array that could not be allocated.  Growing an array synchronises the device (the old one may be in
 // use) and drops the cached graphs (their launches name the old texture).
-constexpr size_t kMaxTextures = 12;   // level widths with an array
+//
+// The arrays are bounded in number and kept until the context is destroyed.  The row sweep's three widths
+// always get one.  The widths of the strip-and-band sweep share kMaxTextures, first come: evicting one costs a
+// device synchronisation and the cached graphs, which calls that alternate between many sizes would pay
+// every time, for gathers worth 8 % of the sweep.
+constexpr int kMaxTextures = 12;
 int hr_ref_texture(hrebsd_ctx *ctx, const float *ref, int R, int h, int w, cudaStream_t st, unsigned long long *tex)
 {
     *tex = 0;
@@ -1573,7 +1578,11 @@ int hr_ref_texture(hrebsd_ctx *ctx, const float *ref, int R, int h, int w, cudaS
     size_t mi = ctx->mtex.size();
     for (size_t i = 0; i < ctx->mtex.size(); ++i)
         if (ctx->mtex[i].w == w) mi = i;
-    if (mi == kMaxTextures) return HREBSD_OK;   // (bounded: further widths go without)
+    if (mi == ctx->mtex.size() && !strip_ok(3, w)) {
+        int others = 0;
+        for (const auto &m : ctx->mtex) others += !strip_ok(3, m.w);
+        if (others >= kMaxTextures) return HREBSD_OK;
+    }
     if (mi == ctx->mtex.size() || ctx->mtex[mi].rows < rows) {
         long long cap_rows = rows > 8LL * h ? rows : 8LL * h;   // room for 8 references from the start
         if (mi < ctx->mtex.size()) {
