@@ -329,9 +329,13 @@ def run_ours(args, rank, world, local_rank):
             return "row sweep, one launch per level/w threads"
         if v == 7:
             return "level in shared memory/512t"
+        if v >= P.TILE_VARIANTS:
+            return {P.FORM_CLUSTER: "level in a cluster's shared memory/512t", P.FORM_STRIPS: "sweep over strips and bands",
+                    P.FORM_PLAIN: "64x32, plain loads"}[v]
         return "x".join(map(str, P.TILE_SHAPES[v])) + f"/{P.TILE_THREADS[v]}t"
     tile_choice = [
         {"level": l, "shape": shape_name(P.hrebsd_get_tile_variant(pipe.ctx, wl["H"] >> l, wl["W"] >> l)),
+         "ran": shape_name(P.hrebsd_level_form(pipe.ctx, l)),
          **({"pinned": True} if tune_ms is None else
             {"ms_per_iteration_by_shape": {shape_name(v): round(float(tune_ms[l, v]), 4)
                                            for v in range(P.TILE_VARIANTS) if np.isfinite(tune_ms[l, v])}})}

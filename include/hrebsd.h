@@ -101,10 +101,12 @@ int hrebsd_device_error(hrebsd_ctx *ctx);
  * results agree to FP32 rounding before the BF16 store. */
 #define HREBSD_OPT_CNN_TC 3
 /* HREBSD_OPT_TEX_GATHER (value 0/1, default 1): the row-sweep demons
- * iteration (tile shapes 5 and 6) reads the four moving-image pixels of each
+ * iteration (tile shapes 5 and 6, and the sweep over strips and bands) reads the
+ * four moving-image pixels of each
  * bilinear sample with one texture gather from a copy of the level's
  * reference images in a CUDA array held by the context (one array per level
- * width, grown when a call needs more rows; growing it synchronises the device
+ * width: the row sweep's three and at most twelve others, first come; grown
+ * when a call needs more rows; growing it synchronises the device
  * and drops the cached graphs); 0 selects plain global loads.  The same four
  * values enter the same arithmetic, so the results are identical.  Levels whose
  * R x h rows exceed the device's texture-gather height, and the
@@ -256,8 +258,9 @@ int hrebsd_demons_register_batch_noalloc(hrebsd_ctx *ctx, const float *ref, cons
  * iteration run as shape 5); shape 5 itself takes this form when the batch has
  * no more pairs than the level has resident CTAs (one pair per CTA: nobody
  * waits), and per-iteration launches otherwise (they re-balance the uneven
- * iteration counts of the pairs after every iteration).  A level without a
- * set or tuned shape runs shape 5 where it applies and shape 0 elsewhere.
+ * iteration counts of the pairs after every iteration; levels of 2^24 pixels
+ * or more run shape 4).  A level without a set or tuned shape takes shape 5
+ * where it applies and shape 0 elsewhere.
  * 7 = the whole level in shared memory (levels of at most 64 x 64 pixels):
  * one CTA of 512 threads per pair holds the field, iterates, applies the stop
  * rule and writes the level's final field, one launch per level (other
@@ -265,8 +268,20 @@ int hrebsd_demons_register_batch_noalloc(hrebsd_ctx *ctx, const float *ref, cons
  * (sigma = 1); other radii always use shape 0.  Every shape computes each
  * output pixel with the same operations in the same order, so the field is
  * the same; only the grouping of the per-tile SSD partials changes (shapes 5
- * and 6 share theirs: same counts, same field). */
+ * and 6 share theirs: same counts, same field).
+ *
+ * At the Gaussian radius 3 a level whose shape was not set by
+ * hrebsd_set_tile_variant (a default or an autotuned one) runs in one of two
+ * further forms in place of its shape where an estimate of their times, from the batch
+ * and level size, says that they are faster: the level in the shared memory of
+ * a thread-block cluster per pair (HREBSD_FORM_CLUSTER: few pairs, small levels),
+ * or, in place of a tile shape, the row sweep over strips of columns and bands of rows
+ * (HREBSD_FORM_STRIPS: any width).  Both sum the SSD of the stop rule as the
+ * shape they stand in for does, so counts and field are that shape's. */
 #define HREBSD_TILE_VARIANTS 8
+#define HREBSD_FORM_CLUSTER 8
+#define HREBSD_FORM_STRIPS 9
+#define HREBSD_FORM_PLAIN 10
 
 /* Autotuner: for each pyramid level of an H x W registration with `params`,
  * time every tile shape on synthetic striped patterns displaced by a small
@@ -275,7 +290,8 @@ int hrebsd_demons_register_batch_noalloc(hrebsd_ctx *ctx, const float *ref, cons
  * launch, then the best of 3 launches of 7 (shape 6) or 8 (shape 7)
  * iterations; shape 6 is reported but never chosen,
  * since the synthetic pairs all run the same number of iterations) and keep, for later
- * registrations of that level size in this context, the shape with the least
+ * registrations of that level size in this context (where none of the two
+ * further forms takes its place, see above), the shape with the least
  * time x (1 + 0.01 log2(4096 / tile area)): smaller tiles carry a 1 % handicap
  * per halving of the area, because the synthetic timing showed a tie where
  * the 64x64 shape was 4 % faster on scan data; shapes 0-6 count 0.005 ms more
@@ -288,10 +304,19 @@ int hrebsd_demons_register_batch_noalloc(hrebsd_ctx *ctx, const float *ref, cons
 int hrebsd_autotune(hrebsd_ctx *ctx, int B, int H, int W, const hrebsd_demons_params *params, float *ms_out,
                     void *stream);
 /* Set (variant 0..HREBSD_TILE_VARIANTS-1) or clear (-1) the tile shape used
- * for levels of size h x w; get returns the current choice (0 if none was set
- * or tuned: the level then runs the default above). */
+ * for levels of size h x w: a shape that is set runs wherever it applies, and
+ * neither of the two further forms takes its place.  get returns the shape that was set
+ * or tuned (0 if none was: the level then takes the default above); what a
+ * level ran in is hrebsd_level_form's answer. */
 int hrebsd_set_tile_variant(hrebsd_ctx *ctx, int h, int w, int variant);
 int hrebsd_get_tile_variant(const hrebsd_ctx *ctx, int h, int w);
+/* The form that level `level` of the context's latest registration ran in (its
+ * last part, where a large batch is processed in parts): a tile shape 0..7 as
+ * above (6 also where shape 5 took its one-launch form), HREBSD_FORM_CLUSTER,
+ * HREBSD_FORM_STRIPS, or HREBSD_FORM_PLAIN (64x32 tiles by plain loads: widths that the
+ * tile copies do not take, caps below two).  EINVAL where that
+ * registration skipped the level or none was made. */
+int hrebsd_level_form(const hrebsd_ctx *ctx, int level);
 
 /* a5 -- rotation fit (Section 2, Eq. 2-5).  The field [B][2][H][W] is
  * sampled bilinearly at the N ROI centres c (index coordinates c - 0.5);

@@ -22,7 +22,7 @@ __all__ = [
     "hrebsd_demons_register_batch", "hrebsd_demons_register_batch_noalloc", "hrebsd_fit_rotation", "hrebsd_remap", "hrebsd_xcf_roi_batch",
     "hrebsd_solve_F", "hrebsd_elastic", "elastic_params", "NORM_DET1", "NORM_TRACTION_FREE", "hrebsd_cnn_save", "hrebsd_cnn_load", "hrebsd_gauss_taps", "hrebsd_strain_stress", "hrebsd_profile_enable", "hrebsd_profile_read", "hrebsd_device_error", "hrebsd_set_option", "OPT_NO_TMA", "OPT_GRAPHS", "OPT_CNN_TC", "OPT_TEX_GATHER", "TILE_VARIANTS",
     "hrebsd_autotune", "hrebsd_probe_fp32_fma", "hrebsd_polar_batch", "hrebsd_tc_selftest", "hrebsd_wait_selftest", "hrebsd_cnn_get_state", "hrebsd_cnn_set_state", "hrebsd_fit_quality", "hrebsd_bandpass_batch", "hrebsd_mean_pattern",
-    "hrebsd_background_batch", "hrebsd_shift_zoom_batch", "hrebsd_ssim_warped", "hrebsd_set_tile_variant", "hrebsd_get_tile_variant", "hrebsd_field_resample", "PROF_CLASSES", "PAIR_CAPPED", "PAIR_NONFINITE", "PAIR_FIT_FAILED",
+    "hrebsd_background_batch", "hrebsd_shift_zoom_batch", "hrebsd_ssim_warped", "hrebsd_set_tile_variant", "hrebsd_get_tile_variant", "hrebsd_level_form", "FORM_CLUSTER", "FORM_STRIPS", "FORM_PLAIN", "hrebsd_field_resample", "PROF_CLASSES", "PAIR_CAPPED", "PAIR_NONFINITE", "PAIR_FIT_FAILED",
 ]
 
 PAIR_CAPPED, PAIR_NONFINITE, PAIR_FIT_FAILED = 1, 2, 4
@@ -122,6 +122,7 @@ def load(build: bool = False):
         "hrebsd_ssim_warped": (i, [vp, vp, vp, vp, vp, i, i, i, vp, vp]),
         "hrebsd_set_tile_variant": (i, [vp, i, i, i]),
         "hrebsd_get_tile_variant": (i, [vp, i, i]),
+        "hrebsd_level_form": (i, [vp, i]),
         "hrebsd_strain_stress": (i, [vp, vp, vp, vp, i, i, C.c_double, C.c_double, C.c_double, C.c_double, i, vp,
                                      vp, vp, vp]),
         "hrebsd_cnn_num_params": (ll, [vp]),
@@ -299,6 +300,7 @@ def elastic_params(g, R, tilt_rad, stiffness=None, ref_idx=None):
 
 
 TILE_VARIANTS = 8
+FORM_CLUSTER, FORM_STRIPS, FORM_PLAIN = 8, 9, 10   # forms of a level besides the tile shapes (hrebsd_level_form)
 # 5: the row sweep; 6: the row sweep with a level's iterations after the first in one launch;
 # 7: the whole level (at most 64 x 64) in shared memory, one launch
 TILE_SHAPES = ((64, 32), (32, 32), (64, 16), (64, 32), (64, 64), ("w", "rows"), ("w", "rows"), ("h", "w"))
@@ -381,6 +383,13 @@ def hrebsd_get_tile_variant(ctx, h, w):
     v = load().hrebsd_get_tile_variant(ctx, h, w)
     if v < 0:
         _chk(v, "hrebsd_get_tile_variant")
+    return v
+
+
+def hrebsd_level_form(ctx, level):
+    v = load().hrebsd_level_form(ctx, level)
+    if v < 0:
+        _chk(v, "hrebsd_level_form")
     return v
 
 

@@ -1841,6 +1841,7 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
         }
     }
 
+    for (int &f : ctx->level_form) f = -1;
     for (int l = start; l >= 0; --l) {
         const int h = H >> l, w = W >> l;
         const int cap = p->max_iters[l];
@@ -1908,6 +1909,8 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
             }
             if (wp.NT && (e = hr_ref_texture(ctx, rl[l], R, h, w, st, &mtex))) return e;
         }
+        ctx->level_form[l] = plan.C ? HREBSD_FORM_CLUSTER : wp.NT ? HREBSD_FORM_STRIPS : use_level ? kLevelVariant
+                             : use_loop ? kLoopVariant : use_strip ? kStripVariant : use_tma ? var : HREBSD_FORM_PLAIN;
         // The launches of one level: list reset, cap x (iteration, control) -- or, in the loop
         // form, iteration 0 and its control, then one launch for the rest --, finalize,
         // prolongation.  Replayed from a cached CUDA graph when possible.
@@ -2180,6 +2183,11 @@ extern "C" int hrebsd_get_tile_variant(const hrebsd_ctx *ctx, int h, int w)
     for (const auto &t : ctx->tune)
         if (t.h == h && t.w == w) return t.var;
     return 0;
+}
+
+extern "C" int hrebsd_level_form(const hrebsd_ctx *ctx, int level)
+{
+    return ctx && level >= 0 && level < 8 && ctx->level_form[level] >= 0 ? ctx->level_form[level] : HREBSD_EINVAL;
 }
 
 extern "C" int hrebsd_autotune(hrebsd_ctx *ctx, int B, int H, int W, const hrebsd_demons_params *p, float *ms_out,

@@ -89,6 +89,7 @@ struct hrebsd_ctx {
     std::vector<hr_graph_entry> graph_cache;
     unsigned long long graph_clock = 0;
     std::vector<hr_tune_entry> tune;
+    int level_form[8] = {-1, -1, -1, -1, -1, -1, -1, -1};   // what the levels of the latest registration ran in, -1: skipped
     std::vector<hr_quadric> quadrics;   // the latest pattern sizes, at most 8
     int *d_err = nullptr;   // device flag: a bounded wait gave up (static device symbol)
     hr_cnn_net *cnn = nullptr;   // learned initialiser (allocated on first use)
