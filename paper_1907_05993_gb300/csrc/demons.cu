@@ -1278,7 +1278,7 @@ constexpr int kVarNT[kTileVariants] = {256, 256, 256, 512, 768, 0, 0, 512};   //
 // The shape that a level's iterations run in, without the cluster form.
 struct LevelShape {
     int var;
-    bool level, strip, tma;
+    bool level, strip, tma, loop;
 };
 
 // The cluster form of a level: CTAs per pair, rows per band, clusters resident at once.
@@ -1321,24 +1321,33 @@ int cluster_active(hrebsd_ctx *ctx, int C, int *out)
     return HREBSD_OK;
 }
 
-// Estimated SM cycles of one iteration of B pairs of h x w, fitted to measured levels of 20 iterations of 1
-// to 600 pairs, 23 x 25 to 256 x 256 pixels (within ~15 %).  The row sweep: 512 / w CTAs per SM, one pair
-// each, a step of 7 rows takes longer the fuller the SM is.  The tiles: the launch of the iteration and of
-// the control kernel, then the tiles' pixels.  The level in one CTA: at most two per SM.
+// Estimated SM cycles of one iteration of B pairs of h x w.  Fitted to levels of 20 iterations, 850 combinations of
+// 30 sizes from 8 x 8 to 1024 x 1244, 1 to 12,000 pairs and with or without a stop rule, each in every form that
+// covers it; nine estimates of ten lie between 17 % below and 9 % above the time (cluster form: 10 and 5).
+//
+// The level in one CTA: at most two per SM, which slow each other down; of an odd share the last runs alone.
+// The row sweep: a step of 7 rows takes longer the fuller the SM is (512 / w CTAs); with more pairs than that,
+// a launch per iteration.  The tiles: the launches of the iteration and of the control kernel, then the
+// whole tiles of the fullest SM, by their pixels; by plain loads, a part per tile and a part per pixel inside.
+// One cost per pixel for all tile shapes took the tuned 64 x 64 tiles for 30 % slower than they are and put the
+// sweep over strips in their place where it takes longer (100 pairs of 480 x 640 with a stop rule: 5.6 -> 7.3 ms).
 float shape_cycles(const hrebsd_ctx *ctx, const LevelShape &s, int B, int h, int w)
 {
-    const float sms = (float)ctx->num_sms;
+    const float sms = (float)ctx->num_sms, px = (float)(h * w);
     if (s.level) {
         const int share = (B + ctx->num_sms - 1) / ctx->num_sms;
-        return (float)((share + 1) / 2) * (2000.0f + 2.45f * (float)(h * w) * (share > 1 ? 2.0f : 1.0f));
+        return 2000.0f + (float)(share / 2) * (4600.0f + 4.25f * px) + (float)(share % 2) * (3800.0f + 2.15f * px);
     }
     if (s.strip) {
-        const float load = (float)B * (float)w / (512.0f * sms);
-        return (float)((h + 12) / 7) * (3500.0f + 2700.0f * fminf(load, 1.0f)) * fmaxf(load, 1.0f) + (load > 1.0f ? 6000.0f : 0.0f);
+        const float load = (float)B * (float)w / (512.0f * sms), steps = (float)((h + 12) / 7);
+        return s.loop ? 4000.0f + steps * (3600.0f + 3900.0f * fmaxf(load - 0.22f, 0.0f))
+                      : 30000.0f + steps * (1500.0f + 5550.0f * load);
     }
+    constexpr float kPx[5] = {3.1f, 3.4f, 3.8f, 3.3f, 2.8f};   // cycles per pixel of a shape's tiles
     const int tx = s.tma ? kVarTX[s.var] : TX, ty = s.tma ? kVarTY[s.var] : TY;
-    const float px = (float)((w + tx - 1) / tx * tx) * (float)((h + ty - 1) / ty * ty);   // whole tiles
-    return (s.tma ? 14000.0f : 18000.0f) + (s.tma ? 3.5f : 4.0f) * (float)B * px / sms;
+    const float items = (float)B * (float)((w + tx - 1) / tx) * (float)((h + ty - 1) / ty);
+    if (s.tma) return 14000.0f + kPx[s.var] * ceilf(items / sms) * (float)(tx * ty);
+    return 14500.0f + 8200.0f * fmaxf(items / sms, 1.0f) + 1.23f * (float)B * px / sms;
 }
 
 // The same for the cluster form: once for every round of resident clusters, the barriers and latencies of
@@ -1358,10 +1367,16 @@ int plan_cluster(hrebsd_ctx *ctx, int B, int h, int w, int group, int tasks, Clu
         const int e = cluster_active(ctx, C, &p.active);
         if (e) return e;
         if (p.active < 1) continue;
-        p.cycles = C > 1 ? 6000.0f + 2.3f * (float)(p.hb * w) : 3200.0f + 1.85f * (float)(p.hb * w);
-        if (group == clu::G_STRIP) p.cycles += 2000.0f + 55.0f * (float)h;
-        else if (group != clu::G_FREE) p.cycles += 2000.0f + 2200.0f * (float)((tasks + 16 * C - 1) / (16 * C));
-        p.cycles *= (float)((B + p.active - 1) / p.active);
+        // by pixels, by rounds of vertical runs over the threads, by what the barriers of C CTAs take
+        const bool one = C == 1;
+        const float px = (float)(p.hb * w), Cf = (float)C;
+        const float runs = (float)(((p.hb + clu::VR - 1) / clu::VR * w + clu::NT - 1) / clu::NT);
+        const float warp_tasks = (float)((tasks + clu::NT / 32 * C - 1) / (clu::NT / 32 * C));
+        if (group == clu::G_FREE) p.cycles = (one ? 3000.0f + 1.3f * px : 3900.0f + 96.0f * Cf + 1.75f * px) + 1600.0f * runs;
+        else if (group == clu::G_STRIP) p.cycles = 3300.0f + 0.75f * px + 3250.0f * runs + 90.0f * (float)h;
+        else if (group == clu::G_LEVEL) p.cycles = (one ? 700.0f + 1.7f * px : 3250.0f + 60.0f * Cf + 2.14f * px) + 1500.0f * runs + 4000.0f * warp_tasks;
+        else p.cycles = (one ? 4200.0f + 1.53f * px : 5050.0f + 150.0f * Cf + 2.19f * px) + 2000.0f * runs + 700.0f * warp_tasks;
+        p.cycles = 1350.0f + p.cycles * (float)((B + p.active - 1) / p.active);
         if (!best->C || p.cycles < best->cycles) *best = p;
     }
     return HREBSD_OK;
@@ -1389,15 +1404,16 @@ int launch_cluster(hrebsd_ctx *ctx, const clu::ClusterArgs &a, const ClusterPlan
 }
 
 // The sweep over strips and bands: threads per CTA, strips, bands.  A band's 12 extra rows and a strip's halo
-// columns are recomputed; a wave of CTAs takes about as long half full as full.  Estimated SM cycles as
-// shape_cycles, fitted to 18 sizes, 23 x 25 to 1244 x 1024 (within ~20 %; the chosen split was the fastest of
-// all, or within 8 % of it, at each).  NT = 0: none.
+// columns are recomputed.  The same estimate: the filling and draining of every round of resident CTAs, then
+// its steps, which take the longer the fuller the SM is (a partly filled last round by its fullest SM); with
+// the regrouped SSD (`regroup`: the threads of its CTAs, 0 where it is not needed) a launch more, d written and
+// read.  NT = 0: none.
 struct WidePlan {
     int NT = 0;
     wide::WideArgs w{};
     float cycles = 0.0f;
 };
-WidePlan plan_wide(const hrebsd_ctx *ctx, int B, int h, int w, bool regroup)
+WidePlan plan_wide(const hrebsd_ctx *ctx, int B, int h, int w, long long regroup)
 {
     WidePlan best;
     for (int NT = 128; NT <= 256; NT *= 2) {
@@ -1409,10 +1425,11 @@ WidePlan plan_wide(const hrebsd_ctx *ctx, int B, int h, int w, bool regroup)
         for (int bands = 1; bands == 1 || (bands <= 64 && h / bands >= 16); ++bands) {
             a.bh = (h + bands - 1) / bands;
             a.bands = (h + a.bh - 1) / a.bh;
-            const long long items = (long long)B * a.strips * a.bands;
-            const int steps = (a.bh + (a.bands > 1 ? 18 : 12)) / 7;
-            const float waves = items <= cap ? 0.75f + 0.25f * (float)items / (float)cap : (float)((items + cap - 1) / cap);
-            const float cycles = waves * (26000.0f + 5900.0f * (float)steps);
+            const long long items = (long long)B * a.strips * a.bands, full = items / cap, rem = items % cap;
+            constexpr float kStep[5] = {0.0f, 4400.0f, 5100.0f, 6350.0f, 7500.0f};   // by 128-thread units on an SM
+            const int units = (int)((rem + ctx->num_sms - 1) / ctx->num_sms) * (NT / 128);
+            const float steps = (float)((a.bh + (a.bands > 1 ? 18 : 12)) / 7);
+            const float cycles = 23000.0f * (float)(full + (rem > 0)) - 8300.0f + steps * (6900.0f * (float)full + kStep[units]);
             if (!best.NT || cycles < best.cycles) {
                 best.NT = NT;
                 best.w = a;
@@ -1420,7 +1437,7 @@ WidePlan plan_wide(const hrebsd_ctx *ctx, int B, int h, int w, bool regroup)
             }
         }
     }
-    if (regroup) best.cycles += 6000.0f + 0.82f * (float)B * (float)(h * w) / (float)ctx->num_sms;
+    if (regroup) best.cycles += 5500.0f + (0.23f * (float)B * (float)(h * w) + 3.85f * (float)regroup) / (float)ctx->num_sms;
     return best;
 }
 
@@ -1872,18 +1889,11 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
         WidePlan wp;
         const int tile_tx = use_tma ? kVarTX[var] : TX, tile_ty = use_tma ? kVarTY[var] : TY;
         if (rad == clu::RAD && cap >= 1 && !ctx->no_tma && !hr_pinned_variant(ctx, h, w)) {
-            const LevelShape shape{var, use_level, use_strip, use_tma};
+            const LevelShape shape{var, use_level, use_strip, use_tma, use_loop};
             // the rule can end the level before the cap: the SSD has to be summed as that shape sums it
             const bool regroup = p->stop_window > 0 && cap > p->stop_window;
             const bool tile = !use_level && !use_strip;
-            float limit = 0.9f * shape_cycles(ctx, shape, B, h, w);
-            // (the estimate for the plain-load tiles is up to 15 % low, that for the TMA-fed ones up to 25 % high;
-            // the sweep's is low, the cluster's high at narrow levels)
-            if (tile && !given && h >= 8 && w >= 8 && (long long)h * w < (1 << 24)) {
-                wp = plan_wide(ctx, B, h, w, regroup);
-                if (wp.NT && wp.cycles < (use_tma ? 0.89f : 1.17f) * limit) limit = fminf(limit, 1.2f * wp.cycles);
-                else wp.NT = 0;
-            }
+            float best = shape_cycles(ctx, shape, B, h, w);
             ca.group = !regroup ? clu::G_FREE : use_level ? clu::G_LEVEL : use_strip ? clu::G_STRIP : use_tma ? clu::G_TILE : clu::G_PLAIN;
             ca.tx = tile ? tile_tx : w;
             ca.ty = tile ? tile_ty : h;
@@ -1893,9 +1903,14 @@ int register_chunk(hrebsd_ctx *ctx, const float *ref, const float *test, const i
             ca.tasks = ca.tiles * (ca.nt / 32);
             if (!regroup || ca.tasks <= clu::MAX_TASKS) {
                 if ((e = plan_cluster(ctx, B, h, w, ca.group, ca.tasks, &plan))) return e;
-                if (plan.C && plan.cycles > limit) plan.C = 0;
+                if (plan.C && plan.cycles < best) best = plan.cycles;
+                else plan.C = 0;
             }
-            if (plan.C) wp.NT = 0;
+            if (tile && !given && h >= 8 && w >= 8 && (long long)h * w < (1 << 24)) {
+                wp = plan_wide(ctx, B, h, w, regroup ? (long long)B * ca.tiles * ca.nt : 0);
+                if (wp.NT && wp.cycles < best) plan.C = 0;
+                else wp.NT = 0;
+            }
             if (wp.NT && regroup) {
                 // no room for d, or no leave to make some (the call's other slots may be large enough already
                 // where this one is not: it is used at some batches and with a stop rule only): the tiles
