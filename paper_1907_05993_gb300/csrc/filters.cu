@@ -9,6 +9,9 @@
 // mean over the scan in FP64).
 #include <math.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace {
@@ -42,7 +45,7 @@ __device__ __forceinline__ float guarded_div(float a, float d) { return fabsf(d)
 
 // One direction of the separable blur (AXIS 0: along x, 1: along y), replicated borders.
 //
-// A CTA takes 32 lines (rows for x, columns for y) and a segment of at most 256 outputs along them; the
+// A CTA takes 32 lines (rows for x, columns for y, of all images one after the other) and a segment of at most 256 outputs along them; the
 // lines lie in shared memory with their halo, two neighbouring lines interleaved as one float2.  Thread
 // (pair, run) computes RUN consecutive outputs of its two lines: the window of RUN inputs sits in
 // registers (input j in slot j mod RUN, so nothing moves), a tap is one shared-memory load and RUN packed
@@ -65,7 +68,7 @@ struct BlurArgs {
     const float *src;   // POST: the image the result is combined with
     const float *bg;    // [H][W] static background (nullable)
     float *out;
-    long long lines;    // rows of all images (x) or columns of one image (y)
+    unsigned lines;     // rows (x) or columns (y; an odd width counts one more, so that a pair is of one image) of all images
     int H, W, segs, seg, stride, vec;   // segments per line, outputs per segment, float2 stride of a line pair
 };
 
@@ -75,10 +78,9 @@ __global__ void __launch_bounds__(256, 3) blur_pass_kernel(BlurArgs a, const __g
     extern __shared__ __align__(16) float2 blur_smem[];
     const int H = a.H, W = a.W, r = f.r, len = AXIS ? H : W;
     const size_t plane = (size_t)H * W;
-    const int s0 = (blockIdx.x % a.segs) * a.seg;            // first output of the segment
-    const long long l0 = (long long)(blockIdx.x / a.segs) * LINES;   // first line
+    const int s0 = (int)(blockIdx.x % a.segs) * a.seg;        // first output of the segment
+    const unsigned l0 = blockIdx.x / a.segs * LINES;          // first line
     const int n_out = min(a.seg, len - s0), n_in = a.seg + 2 * r;
-    const float *img = a.in + (AXIS ? blockIdx.y * plane : 0);
     float *sm = reinterpret_cast<float *>(blur_smem);
     auto slot = [&](int line, int j) { return sm + 2 * ((line >> 1) * a.stride + j) + (line & 1); };
     // asynchronous copies: every load of the tile is in flight at once
@@ -87,16 +89,19 @@ __global__ void __launch_bounds__(256, 3) blur_pass_kernel(BlurArgs a, const __g
                      : "memory");
     };
     if (AXIS) {   // lanes on columns: coalesced loads, conflict-free stores
-        const int line = threadIdx.x & 31, x = (int)l0 + line;
-        if (x < W)
+        const int line = threadIdx.x & 31;
+        const unsigned col = l0 + line, We = (W + 1) & ~1u, image = col / We;
+        const int x = (int)(col - image * We);
+        const float *img = a.in + image * plane + x;
+        if (col < a.lines && x < W)
 #pragma unroll 4
             for (int j = threadIdx.x >> 5; j < n_in; j += (int)blockDim.x >> 5)
-                copy(slot(line, j), img + (size_t)min(max(s0 - r + j, 0), H - 1) * W + x);
+                copy(slot(line, j), img + (size_t)min(max(s0 - r + j, 0), H - 1) * W);
     } else {
         for (int line = threadIdx.x >> 5; line < LINES; line += (int)blockDim.x >> 5) {
-            const long long row = l0 + line;
+            const unsigned row = l0 + line;
             if (row >= a.lines) break;
-            const float *p = img + row * W;
+            const float *p = a.in + (size_t)row * W;
 #pragma unroll 4
             for (int j = threadIdx.x & 31; j < n_in; j += 32)
                 copy(slot(line, j), p + min(max(s0 - r + j, 0), W - 1));
@@ -105,7 +110,7 @@ __global__ void __launch_bounds__(256, 3) blur_pass_kernel(BlurArgs a, const __g
     asm volatile("cp.async.wait_all;" ::: "memory");
     if (PRE)   // every thread divides what it copied
         for (int line = threadIdx.x >> 5; line < LINES; line += (int)blockDim.x >> 5) {
-            const long long row = l0 + line;
+            const unsigned row = l0 + line;
             if (row >= a.lines) break;
             const float *bg = a.bg + (size_t)(row % H) * W;
 #pragma unroll 4
@@ -144,9 +149,10 @@ __global__ void __launch_bounds__(256, 3) blur_pass_kernel(BlurArgs a, const __g
         if (k + u < 2 * r) win[u] = q[k + u + RUN];
     }
     if (AXIS) {
-        const int x = (int)l0 + 2 * pr, rows = live && x < W ? n_out - o0 : 0;   // this thread's outputs
+        const unsigned col = l0 + 2 * pr, We = (W + 1) & ~1u, image = col / We;
+        const int x = (int)(col - image * We), rows = live && col < a.lines ? n_out - o0 : 0;   // this thread's outputs
         const bool two = x + 1 < W;
-        const size_t p0 = (size_t)(s0 + o0) * W + x, at0 = blockIdx.y * plane + p0;
+        const size_t p0 = (size_t)(s0 + o0) * W + x, at0 = image * plane + p0;
         if (POST != POST_NONE) {   // all loads of the run before any use (src may be out: read here, written below)
             float2 c[RUN];
 #pragma unroll
@@ -183,11 +189,29 @@ __global__ void __launch_bounds__(256, 3) blur_pass_kernel(BlurArgs a, const __g
             for (int i = 0; i < RUN; ++i) blur_smem[pr * a.stride + o0 + i] = acc[i];
         __syncthreads();
         for (int line = threadIdx.x >> 5; line < LINES; line += (int)blockDim.x >> 5) {
-            const long long row = l0 + line;
+            const unsigned row = l0 + line;
             if (row >= a.lines) break;
             for (int j = threadIdx.x & 31; j < n_out; j += 32)
-                a.out[row * W + s0 + j] = sm[2 * ((line >> 1) * a.stride + j) + (line & 1)];
+                a.out[(size_t)row * W + s0 + j] = sm[2 * ((line >> 1) * a.stride + j) + (line & 1)];
         }
+    }
+}
+
+// The same pass with one thread per output (no PRE), the same sums in the same order: few or small images, where
+// the chain of a thread's 32 outputs in the kernel above is the time.
+template <int AXIS, int POST>
+__global__ void __launch_bounds__(256) blur_point_kernel(const float *__restrict__ in, const float *src, float *out, size_t total,
+                                                         int H, int W, const __grid_constant__ FilterTaps f)
+{
+    const size_t plane = (size_t)H * W;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        const size_t image = i / plane;
+        const int p = (int)(i - image * plane), y = p / W, x = p - y * W, at = AXIS ? y : x, last = (AXIS ? H : W) - 1;
+        const float *line = in + image * plane + (AXIS ? (size_t)x : (size_t)y * W);
+        float acc = 0.0f;
+#pragma unroll 4
+        for (int k = -f.r; k <= f.r; ++k) acc = fmaf(f.t[k + f.r], __ldg(line + (size_t)min(max(at + k, 0), last) * (AXIS ? W : 1)), acc);
+        out[i] = POST == POST_DIV ? guarded_div(src[i], acc) : POST == POST_SUB ? src[i] - acc : acc;
     }
 }
 
@@ -295,6 +319,28 @@ int grid_of(hrebsd_ctx *ctx, size_t total)
     return (int)(g < cap ? (g ? g : 1) : cap);
 }
 
+// One thread per output while a pass holds little: a tile of the other kernel takes 4 us however little it holds,
+// 10 with divisions, and longer the more taps its threads add in turn; the points take 1.6 us, 0.2 us per million
+// taps and what they move.  The line was drawn through measured times of 1 to 20,000 images of 8 x 8 to
+// 1024 x 1244 (within 25 % of the better one).  Lines shorter than 32 leave most of a tile empty.  Static and
+// dynamic correction, sigma 5, tiles -> points: one image of 92 x 100 30.1 -> 7.8 us, four of 256 x 256 24.3 -> 13.9,
+// 20,000 of 8 x 8 163 -> 44; 30 of 256 x 256 stay with the tiles (29 us, points 74).
+bool by_points(int n, int H, int W, const FilterTaps &f, bool divides)
+{
+    const double px = 1e-6 * n * H * W, taps = 2 * f.r + 1, narrow = std::max(1.0, 32.0 / std::min(H, W));
+    return 0.5 * px * taps + 4.5 * px <= (divides ? (7.9 + 0.06 * taps) * narrow : 1.7 + 0.05 * taps) * narrow;
+}
+
+template <int AXIS, int POST>
+int launch_points(hrebsd_ctx *ctx, const float *in, const float *src, float *out, int n, int H, int W, const FilterTaps &f,
+                  cudaStream_t st)
+{
+    const size_t total = (size_t)n * H * W;
+    blur_point_kernel<AXIS, POST><<<grid_of(ctx, total), 256, 0, st>>>(in, src, out, total, H, W, f);
+    HR_LAUNCHED(ctx);
+    return HREBSD_OK;
+}
+
 template <int AXIS, bool PRE, int POST>
 int launch_pass(hrebsd_ctx *ctx, const float *in, const float *src, const float *bg, float *out, int n, int H, int W,
                 const FilterTaps &f, cudaStream_t st)
@@ -306,8 +352,7 @@ int launch_pass(hrebsd_ctx *ctx, const float *in, const float *src, const float 
     a.out = out;
     a.H = H;
     a.W = W;
-    a.lines = AXIS ? W : (long long)n * H;
-    const int len = AXIS ? H : W;
+    const int len = AXIS ? H : W, per_image = AXIS ? (W + 1) / 2 * 2 : H;   // lines of an image
     a.segs = (len + MAX_SEG - 1) / MAX_SEG;
     const int runs = ((len + a.segs - 1) / a.segs + RUN - 1) / RUN;   // at most 16
     a.seg = runs * RUN;
@@ -316,16 +361,18 @@ int launch_pass(hrebsd_ctx *ctx, const float *in, const float *src, const float 
     const size_t smem = (size_t)PAIRS * a.stride * sizeof(float2);
     auto k = blur_pass_kernel<AXIS, PRE, POST>;
     if (smem > 48 * 1024) HR_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM));
-    const int threads = (runs * PAIRS + 31) / 32 * 32;   // whole warps
-    const long long tiles = (a.lines + LINES - 1) / LINES * a.segs;
-    for (int i0 = 0; i0 < (AXIS ? n : 1); i0 += 65535) {   // y: one image per grid row
+    // (lines are counted in 32 bits: more images than that go in parts)
+    const int part = (int)std::min<long long>(n, std::max(1LL, (1LL << 30) / ((long long)per_image * a.segs)));
+    for (int i0 = 0; i0 < n; i0 += part) {
         const size_t off = (size_t)i0 * H * W;
         BlurArgs c = a;
         c.in += off;
         c.out += off;
         if (c.src) c.src += off;
-        const dim3 grid((unsigned)tiles, AXIS ? (unsigned)(n - i0 < 65535 ? n - i0 : 65535) : 1u);
-        k<<<grid, threads, smem, st>>>(c, f);
+        c.lines = (unsigned)std::min(part, n - i0) * (unsigned)per_image;
+        const unsigned tiles = (c.lines + LINES - 1) / LINES * (unsigned)a.segs;
+        const int threads = (runs * PAIRS + 31) / 32 * 32;   // whole warps
+        k<<<tiles, threads, smem, st>>>(c, f);
         HR_LAUNCHED(ctx);
     }
     return HREBSD_OK;
@@ -351,13 +398,22 @@ extern "C" int hrebsd_bandpass_batch(hrebsd_ctx *ctx, const float *in, int n, in
     cudaStream_t st = hr_stream(stream);
     hr_prof_begin(ctx, st);
     float *x = (float *)t0, *y = (float *)t1;
-    if ((e = launch_pass<0, false, POST_NONE>(ctx, in, nullptr, nullptr, x, n, H, W, lp, st))) return e;
-    if (hp.r > 0 || sigma_hp > 0.0f) {   // out = G_lp * in - G_hp * in (in may be out: read by the x passes only)
-        if ((e = launch_pass<1, false, POST_NONE>(ctx, x, nullptr, nullptr, y, n, H, W, lp, st))) return e;
-        if ((e = launch_pass<0, false, POST_NONE>(ctx, in, nullptr, nullptr, x, n, H, W, hp, st))) return e;
-        if ((e = launch_pass<1, false, POST_SUB>(ctx, x, y, nullptr, out, n, H, W, hp, st))) return e;
+    // a blur of `in` into dst (in may be dst: read by the x pass only); POST: dst = src - blur
+    auto blur = [&](const FilterTaps &f, const float *src, float *dst, auto post) {
+        constexpr int POST = decltype(post)::value;
+        const bool points = by_points(n, H, W, f, false);
+        const int e2 = points ? launch_points<0, POST_NONE>(ctx, in, nullptr, x, n, H, W, f, st)
+                              : launch_pass<0, false, POST_NONE>(ctx, in, nullptr, nullptr, x, n, H, W, f, st);
+        if (e2) return e2;
+        return points ? launch_points<1, POST>(ctx, x, src, dst, n, H, W, f, st)
+                      : launch_pass<1, false, POST>(ctx, x, src, nullptr, dst, n, H, W, f, st);
+    };
+    using None = std::integral_constant<int, POST_NONE>;
+    if (hp.r > 0 || sigma_hp > 0.0f) {   // out = G_lp * in - G_hp * in
+        if ((e = blur(lp, nullptr, y, None()))) return e;
+        if ((e = blur(hp, y, out, std::integral_constant<int, POST_SUB>()))) return e;
     } else {
-        if ((e = launch_pass<1, false, POST_NONE>(ctx, x, nullptr, nullptr, out, n, H, W, lp, st))) return e;
+        if ((e = blur(lp, nullptr, out, None()))) return e;
     }
     hr_prof_end(ctx, PROF_PRE, st);
     return HREBSD_OK;
@@ -392,7 +448,15 @@ extern "C" int hrebsd_background_batch(hrebsd_ctx *ctx, const float *in, int n, 
     if (sigma_dyn > 0.0f && (e = hr_ws(ctx, WS_F0, total * 4, &t0))) return e;
     float *x = (float *)t0;
     hr_prof_begin(ctx, st);
-    if (sigma_dyn > 0.0f) {   // out may be in: the y pass reads each of its pixels just before it writes it
+    if (sigma_dyn > 0.0f && by_points(n, H, W, f, true)) {   // the divided images in out (which may be in)
+        if (static_bg) {
+            div_kernel<<<grid_of(ctx, total), 256, 0, st>>>(in, static_bg, out, total, plane);
+            HR_LAUNCHED(ctx);
+        }
+        const float *cur = static_bg ? out : in;
+        if ((e = launch_points<0, POST_NONE>(ctx, cur, nullptr, x, n, H, W, f, st))) return e;
+        if ((e = launch_points<1, POST_DIV>(ctx, x, cur, out, n, H, W, f, st))) return e;
+    } else if (sigma_dyn > 0.0f) {   // out may be in: the y pass reads each of its pixels just before it writes it
         e = static_bg ? launch_pass<0, true, POST_NONE>(ctx, in, nullptr, static_bg, x, n, H, W, f, st)
                       : launch_pass<0, false, POST_NONE>(ctx, in, nullptr, nullptr, x, n, H, W, f, st);
         if (e) return e;
