@@ -6,7 +6,7 @@
 // family of the demons smoothing), division by the scan's mean pattern
 // (static) and by the pattern's own blur (dynamic), and a Keys cubic resample
 // for the affine correction.  Everything is FP32 with FP32 accumulation (the
-// mean over the scan in FP64).
+// mean over the scan in three FP32 parts with exact carries, combined in FP64).
 #include <math.h>
 
 #include <algorithm>
@@ -230,18 +230,23 @@ __device__ __forceinline__ void two_sum(float &s, float v, float &e)
     s = t;
 }
 
-// Mean over the n images: 32 pixels x 8 groups of images per CTA.  FP64 additions and conversions would
-// bound it (1000 patterns of 256 x 256: 289 us with one thread per pixel, 261 us with this split), so a
+// Mean over the n images: GROUPS groups of images x 256 / GROUPS pixels per CTA.  FP64 additions and conversions
+// would bound it (1000 patterns of 256 x 256: 289 us with one thread per pixel, 261 us in eight groups), so a
 // group sums in three FP32 parts with exact carries, which hold more bits than one FP64 sum, and only the
-// parts and the groups' sums are added in FP64 (49 us; the read alone takes 39).  Sums that leave the range of FP32 (or are not
-// finite) are repeated in FP64.
+// parts and the groups' sums are added in FP64 (49 us; the read alone takes 39).  Sums that leave the range of
+// FP32 (or are not finite) are repeated in FP64.
+template <int GROUPS>
 __global__ void __launch_bounds__(256) mean_pattern_kernel(const float *__restrict__ in, int n, size_t plane, float *out)
 {
-    __shared__ double part[8][32];
-    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-    const size_t p = (size_t)blockIdx.x * 32 + lane;
+    constexpr int PX = 256 / GROUPS;
+    __shared__ double part[GROUPS][PX];
+    const int lane = threadIdx.x % PX, grp = threadIdx.x / PX;
+    const size_t p = (size_t)blockIdx.x * PX + lane;
     double s = 0.0;
-    if (p < plane) {
+    if (GROUPS == 1 && n <= 2) {   // fewer FP64 operations than the parts' combination
+        if (p < plane)
+            for (int i = 0; i < n; ++i) s += __ldg(in + p + (size_t)i * plane);
+    } else if (p < plane) {
         const float *q = in + p;
         float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, e;
         auto add = [&](float v) {
@@ -250,25 +255,27 @@ __global__ void __launch_bounds__(256) mean_pattern_kernel(const float *__restri
             s2 += e;
         };
         int i = grp;
-        for (; i + 56 < n; i += 64) {
+        for (; i + 7 * GROUPS < n; i += 8 * GROUPS) {
             float v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = __ldg(q + (size_t)(i + 8 * j) * plane);
+            for (int j = 0; j < 8; ++j) v[j] = __ldg(q + (size_t)(i + GROUPS * j) * plane);
 #pragma unroll
             for (int j = 0; j < 8; ++j) add(v[j]);
         }
-        for (; i < n; i += 8) add(__ldg(q + (size_t)i * plane));
+        for (; i < n; i += GROUPS) add(__ldg(q + (size_t)i * plane));
         s = (double)s0 + ((double)s1 + (double)s2);
         if (!isfinite(s)) {
             s = 0.0;
-            for (i = grp; i < n; i += 8) s += __ldg(q + (size_t)i * plane);
+            for (i = grp; i < n; i += GROUPS) s += __ldg(q + (size_t)i * plane);
         }
     }
-    part[grp][lane] = s;
-    __syncthreads();
+    if (GROUPS > 1) {
+        part[grp][lane] = s;
+        __syncthreads();
+    }
     if (grp == 0 && p < plane) {
 #pragma unroll
-        for (int g = 1; g < 8; ++g) s += part[g][lane];
+        for (int g = 1; g < GROUPS; ++g) s += part[g][lane];
         out[p] = (float)(s / n);
     }
 }
@@ -427,7 +434,11 @@ extern "C" int hrebsd_mean_pattern(hrebsd_ctx *ctx, const float *in, int n, int 
     cudaStream_t st = hr_stream(stream);
     hr_prof_begin(ctx, st);
     const size_t plane = (size_t)H * W;
-    mean_pattern_kernel<<<(unsigned)((plane + 31) / 32), 256, 0, st>>>(in, n, plane, out);
+    // few images leave the groups little to share, and 32 pixels are little work for a CTA: 1024 x 1244, one image
+    // 156 us in groups, 28 without, 16 images 158 and 99; from 32 images (small planes: 8) the groups are as fast
+    const int groups = n < 8 || (n < 32 && plane >= 32768) ? 1 : 8;
+    const unsigned ctas = (unsigned)((plane * groups + 255) / 256);
+    (groups == 1 ? mean_pattern_kernel<1> : mean_pattern_kernel<8>)<<<ctas, 256, 0, st>>>(in, n, plane, out);
     hr_prof_end(ctx, PROF_PRE, st);
     HR_LAUNCHED(ctx);
     return HREBSD_OK;
