@@ -9,7 +9,9 @@
 // the kernel is bound by instruction issue (16 loads, the weights and 20 FMAs
 // per pixel).  A thread computes ROWS output rows of its column, so that what
 // depends on the pair, the column or the row group is worked out once for
-// them: 2,500 pairs of 256 x 256 1,030 us, one row at a time 1,204 us.
+// them: 2,500 pairs of 256 x 256 1,030 us, one row at a time 1,204 us.  Few
+// pairs take one row per thread: a thread's rows are then the time (one pair
+// of 128 x 128 2.8 us, four rows 4.4).
 #include "internal.cuh"
 
 namespace {
@@ -25,12 +27,11 @@ __device__ __forceinline__ void keys_weights(float t, float *wt)
     wt[3] = ((a * s3 - 5.0f * a) * s3 + 8.0f * a) * s3 - 4.0f * a;
 }
 
-constexpr int ROWS = 4;   // output rows of a thread
-
 // A CTA walks a contiguous run of row groups (ROWS consecutive rows of one pair; all index arithmetic
 // 32-bit), threads along the rows; R^T of a pair is converted to FP32 registers once, when the run enters
 // the pair.  Pixels whose 4 x 4 footprint lies inside the reference read it without clamping; the others
 // clamp every tap (the same values, since the clamp only acts outside).
+template <int ROWS>
 __global__ void __launch_bounds__(256) remap_kernel(const float *__restrict__ ref, const int32_t *__restrict__ ref_idx,
                                                     const double *__restrict__ Rf, int B, int H, int W, float xpc,
                                                     float ypc, float zs, unsigned groups_per_cta, float *__restrict__ out)
@@ -117,12 +118,18 @@ extern "C" int hrebsd_remap(hrebsd_ctx *ctx, const float *ref, const int32_t *re
     const int threads = W >= 256 ? 256 : (W + 31) / 32 * 32;
     const long long cap = (long long)ctx->num_sms * (2048 / threads);   // resident CTAs
     hr_prof_begin(ctx, hr_stream(stream));
-    const long long groups = (long long)B * ((H + ROWS - 1) / ROWS);
+    // rows of a thread: one where the rows fill at most half the chip (four are 4 units of a CTA's time in turn),
+    // four while their groups are resident at once, and then what takes less in whole rounds (four rows take 3.4
+    // times one row's time): 24 pairs of 240 x 320, 1.2 rounds of four rows, 18.7 us by single rows, 23.2 by fours
+    const long long fours = (long long)B * ((H + 3) / 4);
+    auto rounds = [&](long long n) { return (n + cap - 1) / cap; };
+    const bool single = 2 * rows <= cap || (fours > cap && 10 * rounds(rows) < 34 * rounds(fours));
+    const int group = single ? 1 : 4;
+    const long long groups = (long long)B * ((H + group - 1) / group);
     const unsigned grid = (unsigned)(groups < cap ? groups : cap);
     const unsigned per = (unsigned)((groups + grid - 1) / grid);   // row groups of one CTA's run
-    remap_kernel<<<grid, threads, 0, hr_stream(stream)>>>(ref, ref_idx, R_finite, B, H, W, (float)(g->xstar * W),
-                                                          (float)(g->ystar * H), (float)(g->zstar * W), per,
-                                                          remapped);
+    (group == 1 ? remap_kernel<1> : remap_kernel<4>)<<<grid, threads, 0, hr_stream(stream)>>>(
+        ref, ref_idx, R_finite, B, H, W, (float)(g->xstar * W), (float)(g->ystar * H), (float)(g->zstar * W), per, remapped);
     hr_prof_end(ctx, PROF_REMAP, hr_stream(stream));
     HR_LAUNCHED(ctx);
     return HREBSD_OK;
