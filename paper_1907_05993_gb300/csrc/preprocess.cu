@@ -25,6 +25,7 @@
 namespace {
 
 constexpr int kPreThreads = 512, kPreChunk = 8;
+constexpr int kSmallThreads = 128, kSmallDim = 128, kSmallPixels = 4096;   // small patterns (see preprocess_kernel)
 
 struct QuadricInverse {
     double ginv[36];   // inverse Gram matrix of the basis {1, x, y, x^2, xy, y^2}
@@ -219,22 +220,25 @@ __device__ __forceinline__ T remote(const T *p, unsigned r)
 }
 
 // COL: the width divides the CTA's threads, so that a thread's pixels lie in one column.
+// NT threads on patterns of at most DIM rows and columns.  Patterns of up to 4,096 pixels take 128 threads: 512 of
+// them have little to do each and only three such CTAs fit an SM: 20,000 of 8 x 8 1,967 -> 568 us (without the fit
+// 1,444 -> 382), 2,000 of 64 x 64 219 -> 69, one of 64 x 64 22 -> 14.
 // CL: a cluster of CTAs shares the pattern, the chunks dealt out in turn.  The threads' partial sums of the
 // ranks are added exactly (Sum3), thread by thread, in rank 0, so that they are the sums of one CTA.
-template <bool COL, bool CL>
-__global__ void __launch_bounds__(kPreThreads, CL ? 2 : 3) preprocess_kernel(const float *__restrict__ in, float *out, int H,
+template <bool COL, bool CL, int NT = kPreThreads, int DIM = kMaxDim>
+__global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) preprocess_kernel(const float *__restrict__ in, float *out, int H,
                                                                  int W, int flat, QuadricInverse qi)
 {
     extern __shared__ float sums[];   // CL: the threads' partial sums [18][kPreThreads]
     const unsigned csize = CL ? cluster_reg(true) : 1, rank = CL ? cluster_reg(false) : 0;
     __shared__ double red[32 * 6];
     __shared__ double coef[7];   // the quadric's coefficients, the pattern's sum
-    __shared__ float2 rowA[kMaxDim], rowB[kMaxDim];   // per row: c0 + c2 y + c5 y^2 and c1 + c4 y (hi, lo)
-    __shared__ float2 colX[COL ? 1 : kMaxDim];        // per column: x (hi, lo)
-    __shared__ float rowY[kMaxDim];                   // per row: y (the correctly rounded FP32 coordinate)
+    __shared__ float2 rowA[DIM], rowB[DIM];   // per row: c0 + c2 y + c5 y^2 and c1 + c4 y (hi, lo)
+    __shared__ float2 colX[COL ? 1 : DIM];        // per column: x (hi, lo)
+    __shared__ float rowY[DIM];                   // per row: y (the correctly rounded FP32 coordinate)
     const size_t base = (size_t)(CL ? blockIdx.x / csize : blockIdx.x) * H * W;
     const float *img = in + base;
-    constexpr int bd = kPreThreads;
+    constexpr int bd = NT;
     const int t = threadIdx.x;
     auto row_of = [&](int p) { return (int)__umulhi((unsigned)p, qi.mw); };
     const int n = H * W, rstep = COL ? bd / W : 0;   // COL: rows between a thread's pixels
@@ -626,13 +630,16 @@ extern "C" int hrebsd_preprocess_batch(hrebsd_ctx *ctx, const float *in, int n, 
     // 103 -> 98 us in pairs and 147 us in fours; one 128 x 128, of four chunks, 30 -> 32 us
     int C = 8;
     while (C > 1 && ((long long)n * C > 2 * ctx->num_sms || (long long)H * W < 4LL * C * kPreChunk * kPreThreads)) C /= 2;
+    const bool small = C == 1 && H <= kSmallDim && W <= kSmallDim && H * W <= kSmallPixels;
+    const int threads = small ? kSmallThreads : kPreThreads;
     // widths that divide the CTA (64, 128, 256 ...): the column's terms once per thread
-    const bool col = kPreThreads % W == 0;
-    auto k = C > 1 ? (col ? preprocess_kernel<true, true> : preprocess_kernel<false, true>)
+    const bool col = threads % W == 0;
+    auto k = small ? (col ? preprocess_kernel<true, false, kSmallThreads, kSmallDim> : preprocess_kernel<false, false, kSmallThreads, kSmallDim>)
+           : C > 1 ? (col ? preprocess_kernel<true, true> : preprocess_kernel<false, true>)
                    : (col ? preprocess_kernel<true, false> : preprocess_kernel<false, false>);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(n * C));
-    cfg.blockDim = dim3(kPreThreads);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.stream = hr_stream(stream);
     cudaLaunchAttribute at;
     if (C > 1) {
