@@ -655,8 +655,6 @@ int launch_halo_t(hrebsd_ctx *ctx, const ConvArgs &a, cudaStream_t st)
     return HREBSD_OK;
 }
 
-// Halo tiles by TMA into tcgen05 MMAs (forward convolutions with BF16 output and
-// the tiled weight copy).  Returns 1 when the shape is not covered.
 // What the epilogue of a convolution makes of its output besides (or, with `only`, instead of) storing it;
 // `done` tells whether the kernel that ran did so (the tcgen05 forward kernel does).
 struct Fuse {
@@ -668,6 +666,8 @@ struct Fuse {
     bool only = false, done = false;
 };
 
+// Halo tiles by TMA into tcgen05 MMAs (forward convolutions with BF16 output and
+// the tiled weight copy).  Returns 1 when the shape is not covered.
 template <int RES>
 int launch_tma_t(hrebsd_ctx *ctx, const ConvArgs &a, const bf16 *wt, Fuse *fz, cudaStream_t st)
 {

@@ -827,7 +827,6 @@ __global__ void __launch_bounds__(NT_, MINB) demons_iter_tma_kernel(const __grid
     if (tid == 0 && prev_pair >= 0) write_partial();
 }
 
-
 #include "demons_strip.cuh"
 #include "demons_level.cuh"
 #include "demons_cluster.cuh"

@@ -20,9 +20,11 @@
 //
 // The SSD of the stop rule.  Without a stop rule the SSD only tells whether the field stayed finite, and
 // each CTA sums its own pixels.  With one, an SSD that differs in the last FP32 bit can end a level an
-// iteration earlier or later, so the sum is formed exactly as the shape that would run otherwise forms it
-// (`group`): d is kept in shared memory, and warps of the cluster stand in for the warps of that shape's
-// tiles, adding the same pixels in the same order, the same warp tree, and the tiles in FP64.
+// iteration earlier or later, so the tiles' sums are formed exactly as the shape that would run otherwise
+// forms them (`group`): d is kept in shared memory, and warps of the cluster stand in for the warps of that
+// shape's tiles, adding the same pixels in the same order with the same warp tree.  The tiles are added in
+// FP64, by 32 lanes and a tree where the control kernel takes fewer lanes: the sum of up to 1,024 FP32 values is
+// exact in FP64, so the same in any order, unless they differ by more than a factor of 2^19.
 namespace clu {
 
 constexpr int NT = 512, RAD = 3, VR = 4, MAXC = 16, MAX_TASKS = 1024;

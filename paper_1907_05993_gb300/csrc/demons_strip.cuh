@@ -34,7 +34,6 @@ namespace strip {
 
 constexpr int R = 7;
 
-
 template <int RAD, int NT>
 struct Geo {
     static_assert(2 * RAD + 1 == R, "the register windows rotate with the step only for 2r + 1 = R");
