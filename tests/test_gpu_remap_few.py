@@ -34,7 +34,7 @@ def test_a_pair_alone_equals_the_pair_in_a_batch(H, W):
 
 
 def test_one_pair_is_quick():
-    """2.8 us by single rows, 4.4 by four rows per thread."""
+    """2.5 to 2.8 us by single rows, 4.1 to 4.4 by four rows per thread."""
     import torch
     import paper_1907_05993_gb300 as P
     ctx, geom = P.hrebsd_create(0), P.hrebsd_geometry(0.5, 0.5, 0.6)
@@ -54,4 +54,4 @@ def test_one_pair_is_quick():
         b.synchronize()
         best = min(best, a.elapsed_time(b) / 32 * 1e3)
     P.hrebsd_destroy(ctx)
-    assert best <= 3.6, best
+    assert best <= 3.9, best
