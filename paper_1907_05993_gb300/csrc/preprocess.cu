@@ -238,10 +238,10 @@ __global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) prepro
     __shared__ float rowY[DIM];                   // per row: y (the correctly rounded FP32 coordinate)
     const size_t base = (size_t)(CL ? blockIdx.x / csize : blockIdx.x) * H * W;
     const float *img = in + base;
-    constexpr int bd = NT;
+    constexpr int bd = NT, cs = kPreThreads;   // threads; pixels between two of a chunk (whatever the threads: same sums)
     const int t = threadIdx.x;
     auto row_of = [&](int p) { return (int)__umulhi((unsigned)p, qi.mw); };
-    const int n = H * W, rstep = COL ? bd / W : 0;   // COL: rows between a thread's pixels
+    const int n = H * W, rstep = COL ? cs / W : 0;   // COL: rows between a chunk's pixels
 
     // Sums are taken in FP32 over chunks of kChunk pixels of one thread, the chunk sums added exactly and
     // the threads' sums in FP64: the quadric's coefficients come out of a poorly conditioned 6 x 6 system, and plain FP32
@@ -258,19 +258,27 @@ __global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) prepro
         for (int i = t; i < H; i += bd) rowY[i] = pixel_coord(i, H).hi;
         __syncthreads();
     }
-    // f(p0, whole) for the chunks p0, p0 + bd, ... of this thread; whole: every pixel is inside (else f counts
+    // f(p0, whole) for this thread's chunks of the pixels p0, p0 + cs, ...; whole: every pixel is inside (else f counts
     // the others as 0).  A chunk's pixels are loaded before any of them is used, so that a thread has kChunk
     // loads in flight: the passes are bound by memory latency otherwise.
     auto chunks = [&](auto f) {
-        int p0 = t + (int)rank * (kChunk * bd);
-        for (; p0 + (kChunk - 1) * bd < n; p0 += (int)csize * (kChunk * bd)) f(p0, std::true_type());
-        if (p0 < n) f(p0, std::false_type());
+        auto from = [&](int q) {
+            int p0 = q + (int)rank * (kChunk * cs);
+            for (; p0 + (kChunk - 1) * cs < n; p0 += (int)csize * (kChunk * cs)) f(p0, std::true_type());
+            if (p0 < n) f(p0, std::false_type());
+        };
+        if constexpr (bd == cs) from(t);
+        else
+#pragma unroll 1
+            for (int q = t; q < cs; q += bd) from(q);
     };
+    // false for pixels c of a chunk that are past the end for every thread (small patterns)
+    auto any = [&](int c, auto whole) { return bd == cs || whole || c * cs < n; };
     // last: read for the last time (the line is the first to leave L2)
     auto load = [&](const float *src, int p0, auto whole, float (&v)[kChunk], auto last) {
 #pragma unroll
         for (int c = 0; c < kChunk; ++c)
-            v[c] = whole || p0 + c * bd < n ? (last ? __ldcs(src + p0 + c * bd) : src[p0 + c * bd]) : 0.0f;
+            v[c] = whole || p0 + c * cs < n ? (last ? __ldcs(src + p0 + c * cs) : src[p0 + c * cs]) : 0.0f;
     };
     // row and column of a chunk's pixel c (past the end: the last row); i0 = row_of(p0)
     auto cell = [&](int p0, int i0, int c, auto whole, int &i, int &j) {
@@ -279,7 +287,7 @@ __global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) prepro
             if (!whole) i = min(i, H - 1);
             j = 0;
         } else {
-            const int p = whole ? p0 + c * bd : min(p0 + c * bd, n - 1);
+            const int p = whole ? p0 + c * cs : min(p0 + c * cs, n - 1);
             i = c == 0 ? i0 : row_of(p);
             j = p - i * W;
         }
@@ -335,6 +343,7 @@ __global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) prepro
             const int i0 = row_of(p0);
 #pragma unroll
             for (int c = 0; c < kChunk; ++c) {
+                if (!any(c, whole)) break;
                 int i, j;
                 cell(p0, i0, c, whole, i, j);
                 float phi[6];
@@ -440,6 +449,7 @@ __global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) prepro
             const int i0 = row_of(p0);
 #pragma unroll
             for (int c = 0; c < kChunk; c += 2) {   // two pixels at a time
+                if (!any(c, whole)) break;
                 int i, j, i2, j2;
                 cell(p0, i0, c, whole, i, j);
                 cell(p0, i0, c + 1, whole, i2, j2);
@@ -460,10 +470,10 @@ __global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) prepro
                 const float2 r = __ffma2_rn(nq, f.lo, __ffma2_rn(nq, f.hi, vv));
                 const ff2 e = fast_two_sum(q, __fmul2_rn(r, rf));
                 const float2 d = __fadd2_rn(__fadd2_rn(e.hi, both(-K)), e.lo);
-                if (whole || p0 + c * bd < n) o[p0 + c * bd] = d.x;
-                if (whole || p0 + (c + 1) * bd < n) o[p0 + (c + 1) * bd] = d.y;
-                sd += whole || p0 + c * bd < n ? d.x : 0.0f;
-                sd += whole || p0 + (c + 1) * bd < n ? d.y : 0.0f;
+                if (whole || p0 + c * cs < n) o[p0 + c * cs] = d.x;
+                if (whole || p0 + (c + 1) * cs < n) o[p0 + (c + 1) * cs] = d.y;
+                sd += whole || p0 + c * cs < n ? d.x : 0.0f;
+                sd += whole || p0 + (c + 1) * cs < n ? d.y : 0.0f;
             }
             sum_d.add(sd);
         });
@@ -474,8 +484,8 @@ __global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) prepro
 #pragma unroll
             for (int c = 0; c < kChunk; ++c) {
                 const float d = __fadd_rn(__fsub_rn(v[c], K), 0.0f);
-                if (whole || p0 + c * bd < n) {
-                    o[p0 + c * bd] = d;
+                if (whole || p0 + c * cs < n) {
+                    o[p0 + c * cs] = d;
                     sd += d;
                 }
             }
@@ -491,7 +501,7 @@ __global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) prepro
         load(o, p0, whole, v, std::false_type());
 #pragma unroll
         for (int c = 0; c < kChunk; ++c) {
-            const float d = whole || p0 + c * bd < n ? __fsub_rn(v[c], md) : 0.0f;
+            const float d = whole || p0 + c * cs < n ? __fsub_rn(v[c], md) : 0.0f;
             ss = fmaf(d, d, ss);
         }
         sum_v.add(ss);
@@ -504,7 +514,7 @@ __global__ void __launch_bounds__(NT, CL ? 2 : NT == kPreThreads ? 3 : 8) prepro
         load(o, p0, whole, v, std::true_type());
 #pragma unroll
         for (int c = 0; c < kChunk; ++c)
-            if (whole || p0 + c * bd < n) __stcs(o + p0 + c * bd, __fsub_rn(v[c], md) * inv);
+            if (whole || p0 + c * cs < n) __stcs(o + p0 + c * cs, __fsub_rn(v[c], md) * inv);
     });
 }
 
